@@ -55,7 +55,7 @@ cudaError_t run_lambda(const double* a2d, const Geom& g, const double2* stw64, c
                        double* lnat,
                        double* lpb64, float* lpb32, cudaStream_t st);
 // Gohberg-Semencul generator of H' = I + s T(a_0..a_{Np-1}): c' (Np), spectra
-// lam_c, lam_s (bit-reversed, scaled) and border correction G (N x r).
+// lam_c, lam_s (bit-reversed, scaled) and border correction G (N x r, column by column).
 // *status_host receives 0 on success, 1 if the Durbin recursion broke down.
 cudaError_t run_generator(const double* a1, const Geom& g, double s, const double2* stw64, const double2* tw64,
                           double* cgen,
@@ -81,7 +81,7 @@ struct StepTables {
   const T* lpb;        // [(Np+1) * 2 * Np]
   const void* lam_s;   // cx<T>[Np]
   const void* lam_c;   // cx<T>[Np]
-  const T* G;          // [N * r]
+  const T* G;          // [r * N] border correction, column q at G + q N
   const struct Conv3* c3 = nullptr;   // FP32, N' = 2048 .. 8192: three-pass column convolution
 };
 
@@ -152,7 +152,7 @@ struct RegInst {
   const float2* lam_s;  // [N'] natural order, scaled as the bit-reversed tables
   const float2* lam_c;  // [N']
   const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled
-  const float* G;       // [N * r] border correction
+  const float* G;       // [r * N] border correction, column q at G + q N
   float* u_hi;          // state: u = u_hi + u_lo (double-float), u_d = u^n - u^{n-1}
   float* u_lo;
   float* u_d;

@@ -343,7 +343,8 @@ __global__ void k_gauss_jordan(double* M, double* Inv, int r) {
   }
 }
 
-// G = -X_top X_bot^-1  (N x r), FP64 and FP32.
+// G = -X_top X_bot^-1 (N x r), FP64 and FP32, stored column by column
+// (G[q * N + k]): the sweeps read it with neighbouring k in neighbouring lanes.
 __global__ void k_border_G(const double* __restrict__ X, const double* __restrict__ Dinv, Geom g, double* G64,
                            float* G32) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -351,8 +352,9 @@ __global__ void k_border_G(const double* __restrict__ X, const double* __restric
   const int k = idx / g.r, q = idx % g.r;
   double acc = 0.0;
   for (int t = 0; t < g.r; ++t) acc += X[k * g.r + t] * Dinv[t * g.r + q];
-  G64[idx] = -acc;
-  G32[idx] = (float)(-acc);
+  const size_t at = (size_t)q * g.N + k;
+  G64[at] = -acc;
+  G32[at] = (float)(-acc);
 }
 
 // Register-path tables.  tw1: exp(-2 pi i t k1 / Np) at [k1 * TT + t] with

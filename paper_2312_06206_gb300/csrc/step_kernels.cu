@@ -134,16 +134,33 @@ __device__ void gs_core(cx<T>* buf, int nvec, int vs, const Geom& g, const cx<T>
   fft_dit<T>(buf, logNp, nvec, vs, stw);
 }
 
+// The bottom entries of the bordered solves, ybot[q] = (H'^-1 v')[N + q] =
+// Re vhat[N + q] + Im vhat[r - 1 - q], once per vector into the real part of
+// vhat[N + q] (which gs_out reads for nothing else).  Ends with a barrier.
+template <typename T>
+__device__ __forceinline__ void gs_bottom(cx<T>* buf, int nvec, int vs, const Geom& g) {
+  for (int t = threadIdx.x; t < nvec * g.r; t += blockDim.x) {
+    const int v = t / g.r, q = t % g.r;
+    cx<T>* vh = buf + v * vs;
+    vh[sidx<T>(g.N + q)].x += vh[sidx<T>(g.r - 1 - q)].y;
+  }
+  __syncthreads();
+}
+
 // (H^-1 v)[k] for k < N from vhat: Re vhat[k] + Im vhat[Np-1-k] plus the
-// border correction sum_q G[k, q] ybot[q], ybot[q] = (H'^-1 v')[N + q].
+// border correction sum_q G[k, q] ybot[q], ybot from gs_bottom.  For N far
+// below N' the correction is the larger part of a sweep (N = 799: r = 225, as
+// many operations as the four transforms): G is read column by column, 32
+// neighbouring k per warp, and ybot as one broadcast, so that the
+// multiply-adds set its time (N = 799, FP64 step: 2.21 -> 1.61 ms, against G
+// row by row and ybot summed anew for every k; 2 N^2 r = 0.29 G multiply-adds
+// take 0.47 ms of it at the FP64 rate).
 template <typename T>
 __device__ __forceinline__ T gs_out(const cx<T>* vh, int k, const Geom& g, const T* __restrict__ G) {
   T y = vh[sidx<T>(k)].x + vh[sidx<T>(g.Np - 1 - k)].y;
-  for (int q = 0; q < g.r; ++q) {
-    const int kb = g.N + q;
-    const T yb = vh[sidx<T>(kb)].x + vh[sidx<T>(g.Np - 1 - kb)].y;
-    y += __ldg(&G[(size_t)k * g.r + q]) * yb;
-  }
+  const T* Gk = G + k;
+#pragma unroll 4
+  for (int q = 0; q < g.r; ++q) y += __ldg(Gk + (size_t)q * g.N) * vh[sidx<T>(g.N + q)].x;
   return y;
 }
 
@@ -463,6 +480,7 @@ k_rows_solve(const cx<T>* __restrict__ S, const T* __restrict__ u, const T* __re
     }
     __syncthreads();
     gs_core<T>(buf, NR, vs, g, stw, tw, lam_s, lam_c);
+    gs_bottom<T>(buf, NR, vs, g);
     for (int t = threadIdx.x; t < nrows * N; t += blockDim.x) {
       const int v = t / N, k = t % N;
       W[(size_t)(row0 + v) * N + k] = gs_out<T>(buf + v * vs, k, g, G);
@@ -502,6 +520,7 @@ k_cols_solve(const T* __restrict__ W, const T* u_cur, T* u_prev, T* u_next, T* u
   }
   __syncthreads();
   gs_core<T>(buf, CT, vs, g, stw, tw, lam_s, lam_c);
+  gs_bottom<T>(buf, CT, vs, g);
   for (int t = threadIdx.x; t < CT * N; t += blockDim.x) {
     const int c = t % CT, j = t / CT;
     const int i = i0 + c;
@@ -566,6 +585,7 @@ k_rows_gs(const T* __restrict__ WT, T* __restrict__ UT, Geom g, const cx<T>* __r
   }
   __syncthreads();
   gs_core<T>(buf, NR, vs, g, stw, tw, lam_s, lam_c);
+  gs_bottom<T>(buf, NR, vs, g);
   for (int t = threadIdx.x; t < nrows * N; t += blockDim.x) {
     const int v = t / N, j = t % N;
     UT[(size_t)(row0 + v) * N + j] = gs_out<T>(buf + v * vs, j, g, G);

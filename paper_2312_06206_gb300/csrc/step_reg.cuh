@@ -205,8 +205,47 @@ __device__ __forceinline__ void load_freq(float2* x, const float2* sm, int t) {
     x[r] = sm[pad32(F::template freq_index<r>(t))];
   });
 }
+// lanes of the calling thread's row: TT consecutive threads of one warp
+template <int TT>
+__device__ __forceinline__ unsigned row_mask() {
+  if constexpr (TT == 32) return 0xffffffffu;
+  else return ((1u << TT) - 1u) << ((threadIdx.x & 31) / TT * TT);
+}
 __device__ __forceinline__ float real_at(const float2* sm, int k) {
   return reinterpret_cast<const float*>(sm + pad32(k >> 1))[k & 1];
+}
+
+// The solve of one vector from vhat in shared memory (natural order):
+// y[q] = (H^-1 v)[k], k = t + TT q < N: Re vhat[k] + Im vhat[N'-1-k] plus the
+// border correction sum_p G[k, p] ybot[p], ybot[p] = Re vhat[N+p] +
+// Im vhat[r-1-p].  ybot is formed once per vector, in the real part of
+// vhat[N + p] (which nothing else reads), then each lane adds column p of G
+// to all its outputs: its loads of one p are independent and coalesced (rows
+// of G and ybot anew for every k before: N = 399, r = 113, FP32 step: 313 ->
+// 163 us; N = 1023, r = 1, one instance: 103 -> 95 us).  sync: the barrier of the vector's
+// threads.
+template <int LOGL, typename Sync>
+__device__ __forceinline__ void gs_out_reg(float* y, float2* sm, int t, const RegInst& I, Sync sync) {
+  using F = rf::RegFFT<float, LOGL>;
+  const int N = I.N, r = I.r;
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int k = t + F::TT * q;
+    y[q] = k < N ? sm[pad32(k)].x + sm[pad32(F::L - 1 - k)].y : 0.f;
+  });
+  if (r == 0) return;
+  for (int p = t; p < r; p += F::TT) sm[pad32(N + p)].x += sm[pad32(r - 1 - p)].y;
+  sync();
+#pragma unroll 1
+  for (int p = 0; p < r; ++p) {
+    const float yb = sm[pad32(N + p)].x;
+    const float* Gp = I.G + (size_t)p * N;
+    static_for<0, F::E>([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const int k = t + F::TT * q;
+      if (k < N) y[q] += __ldg(Gp + k) * yb;
+    });
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -572,21 +611,15 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   gs_reg<LOGL, true>(x, sm, t, s_tw1, s_tw, I.lam_s, I.lam_c);
   store_nat<LOGL>(x, sm, t);
   __syncwarp();
-  if (!valid) return;
-  // (H^-1 B)[k] = Re vhat[k] + Im vhat[Np-1-k] + sum_q G[k,q] ybot[q],
-  // ybot[q] = Re vhat[N+q] + Im vhat[r-1-q]
-  const int r = I.r;
+  if (!valid) return;   // uniform over the row's threads, one part of a warp
+  float y[F::E];
+  gs_out_reg<LOGL>(y, sm, t, I, [] { __syncwarp(row_mask<F::TT>()); });
   float* wrow = I.W + (size_t)row * I.ld;
-#pragma unroll 2
-  for (int q = 0; q < F::E; ++q) {
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
     const int k = t + F::TT * q;
-    if (k < N) {
-      float y = sm[pad32(k)].x + sm[pad32(Np - 1 - k)].y;
-      for (int qq = 0; qq < r; ++qq)
-        y += __ldg(&I.G[(size_t)k * r + qq]) * (sm[pad32(N + qq)].x + sm[pad32(r - 1 - qq)].y);
-      wrow[k] = y;
-    }
-  }
+    if (k < N) wrow[k] = y[q];
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -647,16 +680,15 @@ __global__ void __launch_bounds__(BLOCK, 3) kr_cols_solve(const __grid_constant_
   store_nat<LOGL>(x, sm, t);
   cp_async_wait_all();
   __syncthreads();
+  float y[F::E];
+  gs_out_reg<LOGL>(y, sm, t, I, [] { __syncthreads(); });
   if (!valid) return;
-  const int r = I.r;
   const int first = I.first;
-#pragma unroll 2
-  for (int q = 0; q < F::E; ++q) {
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
     const int j = t + F::TT * q;
     if (j < N) {
-      float uh = sm[pad32(j)].x + sm[pad32(Np - 1 - j)].y;
-      for (int qq = 0; qq < r; ++qq)
-        uh += __ldg(&I.G[(size_t)j * r + qq]) * (sm[pad32(N + qq)].x + sm[pad32(r - 1 - qq)].y);
+      const float uh = y[q];
       // compensated leapfrog: d^{n+1} = d^n + uhat (d^1 = uhat), u^{n+1} = u^n + d^{n+1}
       // with u = u_hi + u_lo kept as a double-float pair (two-sum)
       const float d = first ? uh : s_d[j * C::CT + c] + uh;
@@ -671,7 +703,7 @@ __global__ void __launch_bounds__(BLOCK, 3) kr_cols_solve(const __grid_constant_
       I.u_lo[idx] = l2 - (h2 - s);
       I.u_d[idx] = d;
     }
-  }
+  });
 }
 
 constexpr int kRowBlock = 128;
