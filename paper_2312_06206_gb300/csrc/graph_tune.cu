@@ -262,12 +262,14 @@ sadi_status sadi_autotune(sadi_ctx** ctxs, int count, int g, int flags) {
       if (st != SADI_OK) return st;
       double ms = 0;
       if ((st = time_group(grp, 5, &ms)) != SADI_OK) return st;
-      if (!reg_path_supported(logNp, prec)) {
-        // coordinate descent over the shared-memory engine's decomposition
-        // (the dense form leaves the y-sweep tile unused); the column
-        // convolution may also run as three passes (kConvThreePass)
+      // the shared-memory engine's decompositions beside the register path,
+      // where the GS form may run on either (explicit tiles)
+      if (prec == SADI_PREC_FP32 && logNp >= kBlkMinLog) {
+        // coordinate descent over the shared-memory engine's decomposition;
+        // the column convolution may also run as three passes (kConvThreePass)
         Tiles t = grp[0]->tiles32;
-        const int nfields = prec == SADI_PREC_FP32 ? 3 : 2;
+        bool tiled = false;
+        const int nfields = 3;
         const int opts[3][5] = {{1, 2, 4, 8, 0}, {kConvThreePass, 1, 2, 4, 8}, {1, 2, 4, 8, 0}};
         for (int f = 0; f < nfields; ++f) {
           for (int v : opts[f]) {
@@ -283,10 +285,11 @@ sadi_status sadi_autotune(sadi_ctx** ctxs, int count, int g, int flags) {
             if (m2 < ms) {
               ms = m2;
               t = tt;
+              tiled = true;
             }
           }
         }
-        cd.t = t;
+        if (tiled) cd.t = t;
         log += std::string(" ") + prec_name(prec) +
                fmt("(tiles %.0f/%.0f/%.0f) %.4f ms", t.rows, t.conv_cols, t.solve_cols, ms);
       } else {

@@ -96,24 +96,25 @@ int log2i(int v) {
   return l;
 }
 
+// rows per slot of the register paths' spectrum (RegInst::lds): from N' = 2048
+// on a multiple of 8, so that the 8-row runs of a cluster stay aligned
+int slot_rows(const sadi::Geom& g) { return g.logNp < kBlkMinLog ? g.N : (g.N + 7) / 8 * 8; }
+
 size_t esize(int prec) { return prec == SADI_PREC_FP64 ? sizeof(double) : sizeof(float); }
 
-// The FFT engine of the context's precision: the register path where it
-// serves that precision (both FP32 forms up to N' = 1024, the dense form's FFT
-// part up to N' = 2048), except that explicit tiles keep the dense form on
-// the shared-memory engine at lengths where the GS form runs there too.  The
-// state's row pitch follows the engine (alloc_state).
+// The FFT engine of the context's precision: the register paths for both FP32
+// forms, except that explicit tiles, which the shared-memory engine alone
+// has, select that engine from N' = 2048 on.
 bool wants_reg_path(const sadi_ctx* c) {
   if (!reg_path_supported(c->g.logNp, c->prec)) return false;
-  return !(c->tiles_explicit && !reg_path_supported(c->g.logNp, SADI_PREC_FP32));
+  return !(c->tiles_explicit && c->g.logNp >= kBlkMinLog);
 }
 
 sadi_status alloc_state(sadi_ctx* c) {
-  // row pitch of the N x N arrays: the FP32 forms on the register path pad
-  // their rows to 128 bytes (16-byte vector accesses in the sweep GEMM's
-  // epilogue and the row kernels), everything else keeps rows of N
-  c->g.ld = (c->prec != SADI_PREC_FP64 && c->reg_path) ? (c->g.N + kPitchAlign - 1) / kPitchAlign * kPitchAlign
-                                                        : c->g.N;
+  // row pitch of the N x N arrays: the FP32 forms pad their rows to 128 bytes
+  // (16-byte vector accesses in the sweep GEMM's epilogue and the row
+  // kernels), FP64 keeps rows of N
+  c->g.ld = c->prec != SADI_PREC_FP64 ? (c->g.N + kPitchAlign - 1) / kPitchAlign * kPitchAlign : c->g.N;
   const size_t nn = (size_t)c->g.ld * c->g.N;
   const size_t es = esize(c->prec);
   cudaError_t e;
@@ -135,8 +136,13 @@ sadi_status alloc_state(sadi_ctx* c) {
   CK(cudaMalloc(&c->phi2, nn * es), "cudaMalloc(phi2)");
   // the FP32 forms start their incremental remainder from an FP64 evaluation
   // (N' <= 4096), which needs the spectrum scratch at double size
+  // (the register paths' slots hold lds >= N rows each)
   const size_t ses = (c->prec != SADI_PREC_FP64 && c->g.Np <= 4096) ? sizeof(double) : es;
-  CK(cudaMalloc(&c->S, (size_t)c->g.N * c->g.Np * 2 * ses), "cudaMalloc(spectrum)");
+  const size_t sbytes = (size_t)c->g.N * c->g.Np * 2 * ses;
+  size_t rbytes = c->prec != SADI_PREC_FP64 ? (size_t)slot_rows(c->g) * c->g.Np * sizeof(float2) : 0;
+  // behind the slots: the bottom entries of the bordered solves
+  if (c->prec == SADI_PREC_FP32 && c->g.r > kBorderInline) rbytes += (size_t)c->g.r * c->g.ld * sizeof(float);
+  CK(cudaMalloc(&c->S, sbytes > rbytes ? sbytes : rbytes), "cudaMalloc(spectrum)");
   CK(cudaMalloc(&c->W, nn * es), "cudaMalloc(sweep)");
   if (c->g.ld != c->g.N) {
     // the padding columns stay zero: no kernel writes them, and the state
@@ -145,9 +151,9 @@ sadi_status alloc_state(sadi_ctx* c) {
     for (void* b : pbufs) CK(cudaMemsetAsync(b, 0, nn * es, c->stream), "zero state");
     CK(cudaStreamSynchronize(c->stream), "zero state");
   }
-  // FP32 forms whose tiles select the three-pass column convolution (the
-  // default at N' = 8192): its buffers and tables (kept once allocated)
-  if (c->prec != SADI_PREC_FP64 && c->tiles32.conv_cols == kConvThreePass) {
+  // FP32 forms whose explicit tiles select the three-pass column convolution:
+  // its buffers and tables (kept once allocated)
+  if (c->prec != SADI_PREC_FP64 && !c->reg_path && c->tiles32.conv_cols == kConvThreePass) {
     const sadi_status s3 = ensure_conv3(c);
     if (s3 != SADI_OK) return s3;
   }
@@ -277,8 +283,8 @@ sadi_status create_impl(int eq, int N, double alpha, double kappa, double tau, c
       {(void**)&c->G64, sizeof(double) * ((size_t)N * g.r + 1)},
       {(void**)&c->G32, sizeof(float) * ((size_t)N * g.r + 1)},
       {(void**)&c->stage, sizeof(double) * nn},
-      {(void**)&c->rtw1, sizeof(float2) * Np},
-      {(void**)&c->rlreg, sizeof(float) * nlpb},
+      {(void**)&c->rtw1, sizeof(float2) * (2 * Np + kTw2)},
+      {(void**)&c->rlreg, sizeof(float) * reg_symbol_elems(g)},
       {(void**)&c->rlamc, sizeof(float2) * Np},
       {(void**)&c->rlams, sizeof(float2) * Np},
       {(void**)&c->wd, sizeof(WdState)},
@@ -443,12 +449,14 @@ sadi_status sadi_set_initial(sadi_ctx* c, const double* phi1, const double* phi2
     // engine applies (N' <= 4096), else FP32 from the hi part
     if (c->g.Np <= 4096) {
       StepTables<double> tb{c->stw64, c->tw64, c->lpb64, c->lams64, c->lamc64, c->G64};
-      CK(launch_remainder<double>(c->g, tb, default_tiles<double>(c->g.Np, c->g.N), c->stage, c->S, c->Chi, c->Clo, st),
+      CK(launch_remainder<double>(c->g, tb, default_tiles<double>(c->g.Np, c->g.N), c->stage, N, c->S, c->Chi, c->Clo,
+                                  st),
          "starting remainder");
     } else {
       StepTables<float> tb{c->stw32, c->tw32, c->lpb32, c->lams32, c->lamc32, c->G32, c3_of(c)};
-      CK(launch_remainder<float>(c->g, tb, default_tiles<float>(c->g.Np, c->g.N), static_cast<const float*>(c->ubuf[0]),
-                                 c->S, c->Chi, c->Clo, st),
+      Tiles tl = default_tiles<float>(c->g.Np, c->g.N);
+      if (!c->c3.ZE) tl.conv_cols = 1;   // the three-pass buffers exist for explicit tiles only
+      CK(launch_remainder<float>(c->g, tb, tl, static_cast<const float*>(c->ubuf[0]), ld, c->S, c->Chi, c->Clo, st),
          "starting remainder");
     }
   }
@@ -515,16 +523,20 @@ RhsParams rhs_of(const sadi_ctx* c, long long n) {
 RegInst reg_inst(const sadi_ctx* c) {
   RegInst r{};
   r.tw1 = c->rtw1;
+  r.tw2 = c->rtw1 + c->g.Np;
+  r.tw1h = r.tw2 + kTw2;
   r.tw = c->tw32;
   r.lam_s = c->rlams;
   r.lam_c = c->rlamc;
-  r.lreg = c->rlreg;
+  r.lreg = r.lnat = c->rlreg;
   r.G = c->G32;
   r.u_hi = static_cast<float*>(c->ubuf[0]);
   r.u_d = static_cast<float*>(c->ubuf[1]);
   r.u_lo = c->ulo;
   r.phi2 = static_cast<const float*>(c->phi2);
   r.S = static_cast<float2*>(c->S);
+  r.lds = slot_rows(c->g);
+  r.YB = reinterpret_cast<float*>(r.S + (size_t)r.lds * c->g.Np);
   r.W = static_cast<float*>(c->W);
   r.N = c->g.N;
   r.ld = c->g.ld;
@@ -1025,28 +1037,24 @@ sadi_status sadi_set_tiles(sadi_ctx* c, int rows, int conv_cols, int solve_cols)
   if (dflt) t = f64 ? default_tiles<double>(c->g.Np, c->g.N) : default_tiles<float>(c->g.Np, c->g.N);
   const bool ok = f64 ? tiles_valid<double>(c->g, t) : tiles_valid<float>(c->g, t);
   if (!ok) return fail(c, SADI_EINVAL, "tile sizes invalid for this N and precision");
-  // the engine these tiles select (the dense form at N' = 2048: explicit
-  // tiles the shared-memory engine, the defaults the register path); the
-  // FP64 path's tiles leave the FP32 forms' choice alone
+  // the engine these tiles select (from N' = 2048 on: explicit tiles the
+  // shared-memory engine, the defaults the register path; both keep the state
+  // in the same layout); the FP64 path's tiles leave the FP32 forms' choice
+  // alone
   const bool was_explicit = c->tiles_explicit;
   const bool expl = f64 ? was_explicit : !dflt;
   c->tiles_explicit = expl;
   const bool reg = wants_reg_path(c);
   c->tiles_explicit = was_explicit;
-  if (!f64 && t.conv_cols == kConvThreePass && (reg || !conv3_supported(c->g.logNp)))
+  if (!f64 && !dflt && t.conv_cols == kConvThreePass && (reg || !conv3_supported(c->g.logNp)))
     return fail(c, SADI_EINVAL, "the three-pass convolution serves FFT lengths 2048 .. 8192");
-  if (reg != c->reg_path) {
-    if (c->initialized || c->F)
-      return fail(c, SADI_ESTATE,
-                  "tiles that change the FFT engine (dense form, N' = 2048) must precede sadi_set_initial and "
-                  "sadi_set_source");
-    c->tiles_explicit = expl;
-    c->reg_path = reg;
-    const sadi_status sa = alloc_state(c);
-    if (sa != SADI_OK) return sa;
-  }
+  if (reg != c->reg_path && is_dense(c) && c->g.logNp == kBlkMinLog && (c->initialized || c->F))
+    return fail(c, SADI_ESTATE,
+                "tiles that change the FFT engine (dense form, N' = 2048) must precede sadi_set_initial and "
+                "sadi_set_source");
+  c->reg_path = reg;
   c->tiles_explicit = expl;
-  if (!f64 && t.conv_cols == kConvThreePass) {
+  if (!f64 && !reg && t.conv_cols == kConvThreePass) {
     const sadi_status s3 = ensure_conv3(c);
     if (s3 != SADI_OK) return s3;
   }

@@ -20,7 +20,8 @@ struct Geom {
   int N, Np, logNp, P, logP, r;
   // row pitch (elements) of the context's N x N arrays (state, sweep scratch,
   // phi2, source, remainder pair): N for FP64, N rounded up to a multiple of
-  // kPitchAlign for the FP32 forms (aligned rows for vector accesses)
+  // kPitchAlign for the FP32 forms on either engine (aligned rows for vector
+  // accesses; explicit tiles may change the engine without re-laying the state)
   int ld;
 };
 constexpr int kPitchAlign = 32;
@@ -143,22 +144,30 @@ bool tiles_valid(const Geom& g, const Tiles& t);
 template <typename T>
 cudaError_t step_setup_attributes();
 
-// FP32 register-FFT path (FFT length N' <= 1024; N' = 2048 for the dense
-// form's FFT part).  One instance of a batch:
+// FP32 register-FFT paths: a row per part of a warp up to N' = 1024
+// (step_reg.cuh), per block from 2048 on (step_blk.cuh).  One instance of a
+// batch:
 // natural-order tables and the in-place double-float state.
 struct RegInst {
-  const float2* tw1;    // [N'] two-level FFT twiddles exp(-2 pi i t k1 / N') at [k1 * TT + t]
+  // [N'] first-level FFT twiddles exp(-2 pi i t k1 / N') at [k1 * T + t], T
+  // threads per vector (T = TT of regfft.cuh, or of blkfft.cuh from N' = 2048 on)
+  const float2* tw1;
+  const float2* tw2;    // second-level twiddles of blkfft.cuh at [k2 * R3 + t'] (N' >= 2048)
+  const float2* tw1h;   // [N'] tw1 at half frequencies: exp(-2 pi i t (k1 + 1/2) / N') (N' >= 2048)
   const float2* tw;     // [2N'] exp(-2 pi i k / 2N')
   const float2* lam_s;  // [N'] natural order, scaled as the bit-reversed tables
   const float2* lam_c;  // [N']
-  const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled
+  const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled (N' <= 1024)
+  const float* lnat;    // [(N'+1) * (N'+1)] symbol by x- and y-frequency 0 .. N', scaled (N' >= 2048)
   const float* G;       // [r * N] border correction, column q at G + q N
   float* u_hi;          // state: u = u_hi + u_lo (double-float), u_d = u^n - u^{n-1}
   float* u_lo;
   float* u_d;
   const float* phi2;
-  float2* S;            // spectrum scratch, slot-major: N' slots x N rows (S[k * N + row])
-  float* W;             // N x N sweep scratch
+  float2* S;            // spectrum scratch, slot-major: S[k * lds + row]
+  int lds;              // rows per slot, N rounded up to 8 (64-byte runs of a cluster's rows stay aligned)
+  float* W;             // N x N sweep scratch (by columns between the GS sweeps from N' = 2048 on)
+  float* YB;            // bottom entries of the sweeps' bordered solves, r x ld (r > kBorderInline)
   const float* F;       // optional source field (N x N) or nullptr
   float* C_hi;          // incremental remainder -kappa tau^2 L_h u^n (double-float)
   float* C_lo;
@@ -178,6 +187,9 @@ struct RegInst {
   int eq;               // 0 wave, 1 diffusion (RhsParams::eq); tau2 = tau^2 or tau
 };
 constexpr int kMaxBatch = 32;
+// border ranks up to which the sweep kernels add the border correction
+// themselves (above: border.cuh, one more launch per sweep)
+constexpr int kBorderInline = 32;
 // passed by value as a __grid_constant__ kernel parameter (about 4 KB)
 struct RegBatch {
   int count;
@@ -192,7 +204,14 @@ bool reg_path_supported(int logNp, int prec);
 // W and its BF16 split to Bh / Bl; the sweeps are left to the GEMMs.
 cudaError_t launch_step_reg(const RegBatch& b, int logNp, int max_n, cudaStream_t st, cudaEvent_t* ev,
                             bool dense = false);
-// natural-order FP32 tables of the register path from the FP64 setup products
+// natural-order FP32 tables of the register paths from the FP64 setup
+// products: tw1 (N' entries) followed by tw2 (kTw2) and tw1h (N'), and the symbol
+// (reg_symbol_elems floats: RegInst::lreg or ::lnat by FFT length)
+constexpr int kTw2 = 256;
+constexpr int kBlkMinLog = 11;   // first log2 N' of the block-wide FFT
+inline size_t reg_symbol_elems(const Geom& g) {
+  return g.logNp >= kBlkMinLog ? (size_t)(g.Np + 1) * (g.Np + 1) : (size_t)(g.Np + 1) * 2 * g.Np;
+}
 cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, const double2* lamc64,
                            const double2* lams64, float2* tw1, float* lreg, float2* lamc_nat, float2* lams_nat,
                            cudaStream_t st);
@@ -210,12 +229,12 @@ template <typename T>
 cudaError_t launch_step(const Geom& g, const StepTables<T>& tb, const Tiles& tl, const RhsParams& rp, const T* u_cur,
                         T* u_prev, T* u_next, T* u_lo, const T* phi2, void* S, T* W, cudaStream_t st,
                         cudaEvent_t* ev = nullptr, float* Ch = nullptr, float* Cl = nullptr);
-// C = -kappa tau^2 L_h u (N x N) into the double-float pair (Ch, Cl): the
+// C = -kappa tau^2 L_h u (N x N, row pitch ldu) into the double-float pair (Ch, Cl): the
 // starting value of the incremental remainder (T = double gives it to FP64
 // accuracy; needs the FP64 engine, N' <= 4096).
 template <typename T>
-cudaError_t launch_remainder(const Geom& g, const StepTables<T>& tb, const Tiles& tl, const T* u, void* S, float* Ch,
-                             float* Cl, cudaStream_t st);
+cudaError_t launch_remainder(const Geom& g, const StepTables<T>& tb, const Tiles& tl, const T* u, int ldu, void* S,
+                             float* Ch, float* Cl, cudaStream_t st);
 
 // Dense-inverse form on the shared-memory engine (FP32): row FFT of the
 // increment d, column convolution, incremental remainder and B^n (events

@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "blkfft.cuh"
 #include "fft.cuh"
 #include "sadi_internal.h"
 
@@ -357,28 +358,44 @@ __global__ void k_border_G(const double* __restrict__ X, const double* __restric
   G32[at] = (float)(-acc);
 }
 
-// Register-path tables.  tw1: exp(-2 pi i t k1 / Np) at [k1 * TT + t] with
-// TT = 2^floor(logNp/2); lreg[(k1 * 2 + h) * Np + m] = scale * Lambda(k1, 2m + h)
-// (natural order, k2 folded into [0, Np]); lam*_nat[k] = lam*[brev(k)].
-__global__ void k_reg_tables(Geom g, const double* __restrict__ lnat, double scale,
+// Register-path tables.  tw1: exp(-2 pi i t k1 / Np) at [k1 * T + t] (T: threads
+// per vector), from N' = 2048 on followed by tw2, exp(-2 pi i t' k2 / T) at
+// [k2 * R3 + t'], and tw1h, exp(-2 pi i t (k1 + 1/2) / Np) at [k1 * T + t].  Symbol, scaled: up to N' = 1024 lreg[(k1 * 2 + h) * Np + m] =
+// Lambda(k1, 2m + h) (k2 folded into [0, Np]), above lnat32[k1 * (Np + 1) + k2].
+// lam*_nat[k] = lam*[brev(k)].
+__global__ void k_reg_tables(Geom g, const double* __restrict__ lnat, double scale, int T, int R3,
                              const double2* __restrict__ lamc64, const double2* __restrict__ lams64, float2* tw1,
                              float* lreg, float2* lamc_nat, float2* lams_nat) {
   const int Np = g.Np, logNp = g.logNp, P = g.P;
-  const int logT = logNp / 2;
-  const int TT = 1 << logT;
-  const size_t nl = (size_t)(Np + 1) * 2 * Np;
+  const bool folded = R3 > 0;
+  const size_t nl = folded ? (size_t)(Np + 1) * (Np + 1) : (size_t)(Np + 1) * 2 * Np;
   const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (idx < (size_t)Np) {
     const int k = (int)idx;
-    const int t = k & (TT - 1), k1 = k >> logT;
+    const int t = k % T, k1 = k / T;
     double sn, cs;
     sincospi(2.0 * (double)((long long)t * k1 % Np) / (double)Np, &sn, &cs);
     tw1[k] = make_float2((float)cs, (float)-sn);
+    if (folded) {
+      sincospi((double)((long long)t * (2 * k1 + 1) % P) / (double)Np, &sn, &cs);
+      tw1[Np + kTw2 + k] = make_float2((float)cs, (float)-sn);
+    }
     const double2 a = lamc64[brev(k, logNp)], b = lams64[brev(k, logNp)];
     lamc_nat[k] = make_float2((float)a.x, (float)a.y);
     lams_nat[k] = make_float2((float)b.x, (float)b.y);
   }
+  if (folded && idx < (size_t)T) {
+    const int k = (int)idx;
+    const int t = k % R3, k2 = k / R3;
+    double sn, cs;
+    sincospi(2.0 * (double)(t * k2) / (double)T, &sn, &cs);
+    tw1[Np + k] = make_float2((float)cs, (float)-sn);
+  }
   if (idx < nl) {
+    if (folded) {
+      lreg[idx] = (float)(scale * lnat[idx]);
+      return;
+    }
     const int m = (int)(idx % Np);
     const int h = (int)((idx / Np) % 2);
     const int k1 = (int)(idx / (2 * (size_t)Np));
@@ -446,8 +463,21 @@ cudaError_t launch_stage_twiddles(double2* stw64, float2* stw32, int logL, cudaS
 cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, const double2* lamc64,
                            const double2* lams64, float2* tw1, float* lreg, float2* lamc_nat, float2* lams_nat,
                            cudaStream_t st) {
-  const size_t nl = (size_t)(g.Np + 1) * 2 * g.Np;
-  k_reg_tables<<<nblk(nl, 256), 256, 0, st>>>(g, lnat, scale, lamc64, lams64, tw1, lreg, lamc_nat, lams_nat);
+  const size_t nl = reg_symbol_elems(g);
+  int T = 1 << (g.logNp / 2), R3 = 0;
+  auto blk = [&](auto f) {
+    using F = decltype(f);
+    static_assert(F::T <= kTw2, "room for tw2");
+    T = F::T;
+    R3 = F::R3;
+  };
+  switch (g.logNp) {
+    case 11: blk(bf::BlkFFT<11>{}); break;
+    case 12: blk(bf::BlkFFT<12>{}); break;
+    case 13: blk(bf::BlkFFT<13>{}); break;
+    default: break;
+  }
+  k_reg_tables<<<nblk(nl, 256), 256, 0, st>>>(g, lnat, scale, T, R3, lamc64, lams64, tw1, lreg, lamc_nat, lams_nat);
   return cudaGetLastError();
 }
 

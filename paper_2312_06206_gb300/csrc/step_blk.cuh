@@ -1,0 +1,624 @@
+// step_blk.cuh -- the FP32 S-ADI step (Sec. 3, eq. "ADI scheme equivalent")
+// for FFT lengths N' = 2048 .. 8192 on the block-wide register FFT of
+// blkfft.cuh.  The four kernels of step_reg.cuh, with one row, column half or
+// column per T = 128 or 256 threads:
+//   kb_rows_r2c    row of the increment d^n -> half spectrum along x
+//   kb_cols_conv   x frequency: y FFT (even / odd half) x symbol, inverse
+//   kb_rows_solve  inverse real FFT, C += conv(d^n), B^n, then the x sweep
+//                  (Algorithm 1), or B^n alone (dense-inverse form)
+//   kb_cols_solve  y sweep (Algorithm 1) + compensated leapfrog
+//
+// Between the row and the column kernels the data changes direction twice:
+// the spectrum is stored by x frequency (S[k * lds + row]) and the x sweep's
+// result by column (W[k * ld + row]), so that each column kernel reads one
+// contiguous vector.  A single row would then move 8- or 4-byte pieces a
+// column apart; the rows of a cluster of V = 8 blocks are therefore exchanged
+// through distributed shared memory: block c of the cluster gathers
+// frequencies (columns) c L/V .. of all V rows and moves runs of V rows, 64 or
+// 32 bytes.  This replaces the two transpose passes of the shared-memory
+// engine's y sweep and its 8-byte column gathers.
+//
+// Measured against the shared-memory engine (us per launch, GB300): N = 4095
+// row FFT 145 -> 94, convolution 407 -> 193, B^n 258 -> 177, GS rows 537 ->
+// 365, y sweep 488 (with its transposes) -> 290; N = 8191 row FFT 681 -> 418,
+// convolution 1822 (three passes) -> 1103, GS rows 2649 -> 1921, y sweep 2241
+// -> 1263; N = 2047, four instances: 80 + 192 + 264 -> 75 + 175 + 170 against
+// the 64-elements-per-lane kernels this replaces there.  Instructions per
+// element and transform fell from 134 to about 50; what bounds the kernels now
+// is the latency of the table loads and barriers at 16 to 32 warps per SM
+// (issue 50%, L1 55%, FP32 pipe 38% in the convolution).
+#pragma once
+#include <cuda_runtime.h>
+
+#include "bf16split.cuh"
+#include "blkfft.cuh"
+#include "border.cuh"
+#include "sadi_internal.h"
+
+namespace sadi {
+namespace blk {
+
+using bf::BlkFFT;
+using rf::static_for;
+
+constexpr int kCluster = 8;   // V
+
+// g(u) in full FP32 precision; the general form out of line
+static __device__ __noinline__ float g_general_b(float u, float c1, float c3, float cs) {
+  return (c1 + c3 * u * u) * u + cs * sinf(u);
+}
+__device__ __forceinline__ float g_of_b(const RegInst& I, float u) {
+  if (I.gkind == 1) return -u * u * u;
+  if (I.gkind == 2) return -sinf(u);
+  if (I.gkind == 3) return g_general_b(u, I.gc1, I.gc3, I.gcs);
+  return 0.f;
+}
+
+// Loads of streamed data (read once) that leave L1 to the twiddle, symbol and
+// spectral tables, which every block of the SM reads again.
+__device__ __forceinline__ float2 ld_stream(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_stream(const float* p) {
+  float v;
+  asm volatile("ld.global.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+
+// ---- cluster exchange ---------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
+}
+// Execution barrier of the cluster without the release fence (about 700
+// cycles): enough where only this block's own reads have to be over before
+// its peers write (the block barrier in front completes them).
+__device__ __forceinline__ void cluster_join() {
+  __syncthreads();
+  cluster_arrive_relaxed();
+  cluster_wait();
+}
+// address of p (this block's shared memory) in block `rank` of the cluster
+__device__ __forceinline__ unsigned peer(const void* p, int rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_peer(unsigned a, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_peer(unsigned a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+template <int LOGL>
+struct Cfg {
+  using F = BlkFFT<LOGL>;
+  static constexpr int V = kCluster;
+  static constexpr int SEG = F::L / V;               // frequencies (columns) per block of the exchange
+  static constexpr int QS = F::E / V;                // registers q per segment: t + T q lies in segment q / QS
+  static_assert(SEG % F::T == 0 && QS * V == F::E, "whole register groups per segment");
+  // row pitches of the exchange buffers: a half-warp (8-byte) or a warp
+  // (4-byte) reading V rows x 16/V (32/V) neighbours finds distinct banks
+  static constexpr int P2 = SEG + 16 / V, P1 = SEG + 32 / V;
+  static_assert(V * P2 <= F::BUF && V * P1 <= 2 * F::BUF, "exchange buffers inside the transform buffer");
+  static constexpr size_t bytes = (size_t)F::BUF * sizeof(float2);
+  static constexpr size_t bytes_conv = 2 * bytes;
+  // resident blocks promised to the compiler (its register budget), measured
+  // at N = 4095 (us per launch at 2 / 3 / 4 blocks of 256 threads): r2c 109 /
+  // 100 / 94, dense B^n 208 / 179 / 177, GS rows 378 / 362 / -, columns
+  // 289 / 312, convolution 193 (one block of 512 threads, 128 registers)
+  // against 219 (two, 64 registers).  E = 32 (N' = 8192) needs 128 registers.
+  static constexpr int kM = LOGL == 11 ? 2 : 1;   // half the threads per block
+  static constexpr int kR2cBlocks = LOGL == 13 ? 2 : 4 * kM;
+  static constexpr int kDenseBlocks = LOGL == 13 ? 2 : 4 * kM;
+  static constexpr int kGsBlocks = LOGL == 13 ? 2 : 3 * kM;
+  static constexpr int kColsBlocks = 2 * kM;
+  static constexpr int kConvBlocks = kM;
+};
+
+__device__ __forceinline__ void pdl_allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ---------------------------------------------------------------------------
+template <int LOGL>
+__global__ void __launch_bounds__(BlkFFT<LOGL>::T, Cfg<LOGL>::kR2cBlocks)
+kb_rows_r2c(const __grid_constant__ RegBatch B) {
+  using F = BlkFFT<LOGL>;
+  using C = Cfg<LOGL>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* sm = reinterpret_cast<float2*>(smem_raw);
+  pdl_allow_dependents();
+  const RegInst& I = B.in[blockIdx.y];
+  const int N = I.N, t = threadIdx.x;
+  const int rank = blockIdx.x % C::V, row0 = blockIdx.x - rank, row = blockIdx.x;
+  if (row0 >= N) return;   // the whole cluster
+  const bool valid = row < N;
+  auto sync = [] { __syncthreads(); };
+  pdl_wait_prerequisites();
+  // z[n] = d[2n] + i d[2n+1], zero from n = N'/2 on (2n < N <= N'); an even
+  // offset in a 128-byte aligned row: 8-byte loads, row padding beyond N - 1
+  const float* ur = I.u_d + (size_t)(valid ? row : 0) * I.ld;
+  float2 x[F::E];
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    float2 v = make_float2(0.f, 0.f);
+    if constexpr (q < F::E / 2) {
+      const int n = t + F::T * q;
+      if (valid && 2 * n < N) v = ld_stream(reinterpret_cast<const float2*>(ur + 2 * n));
+      if (2 * n + 1 >= N) v.y = 0.f;
+    }
+    x[q] = v;
+  });
+  F::fwd(x, sm, t, I.tw1, false, I.tw2, sync);
+  static_for<0, F::E>([&](auto qc) { sm[t + F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
+  sync();
+  // X[k] = (Z[k] + conj Z[-k]) / 2 + w^k (Z[k] - conj Z[-k]) / (2 i); slot 0 = X[0] + i X[N']
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int k = t + F::T * q;
+    const float2 Z = x[q], Zc = cconj(sm[(F::L - k) & (F::L - 1)]);
+    const float2 Ev = cscale(cadd(Z, Zc), 0.5f);
+    const float2 Ov = cscale(cmul_mi(csub(Z, Zc)), 0.5f);
+    x[q] = (q == 0 && t == 0) ? make_float2(Ev.x + Ov.x, Ev.x - Ov.x) : cadd(Ev, cmul(__ldg(&I.tw[k]), Ov));
+  });
+  cluster_join();   // every block of the cluster has read its buffer
+  static_for<0, C::V>([&](auto cc) {
+    constexpr int c = decltype(cc)::value;
+    const unsigned dst = peer(sm + rank * C::P2 + t, c);
+    static_for<0, C::QS>([&](auto jc) {
+      constexpr int j = decltype(jc)::value;
+      st_peer(dst + (unsigned)(F::T * j * sizeof(float2)), x[c * C::QS + j]);
+    });
+  });
+  cluster_sync();   // the rows' segments have arrived
+  const int vv = t % C::V, s0 = t / C::V;
+  if (row0 + vv >= N) return;
+  float2* col = I.S + (size_t)(rank * C::SEG + s0) * I.lds + row0 + vv;
+  const float2* src = sm + vv * C::P2 + s0;
+#pragma unroll 4
+  for (int i = 0; i < F::E; ++i) col[(size_t)(F::T / C::V * i) * I.lds] = src[F::T / C::V * i];
+}
+
+// ---------------------------------------------------------------------------
+// Block: x frequency kx = blockIdx.x (0 .. N'); threads 0 .. T-1 the even y
+// frequencies 2 m, T .. 2T-1 the odd ones 2 m + 1.  Frequencies 0 and N' are
+// the real and the imaginary part of slot 0: two blocks, each reading and
+// writing its own halves of the slot's elements.
+template <int LOGL>
+__global__ void __launch_bounds__(2 * BlkFFT<LOGL>::T, Cfg<LOGL>::kConvBlocks)
+kb_cols_conv(const __grid_constant__ RegBatch B) {
+  using F = BlkFFT<LOGL>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_allow_dependents();
+  const RegInst& I = B.in[blockIdx.y];
+  const int N = I.N, kx = blockIdx.x;
+  const int h = threadIdx.x / F::T, t = threadIdx.x % F::T;
+  float2* const sm0 = reinterpret_cast<float2*>(smem_raw);
+  float2* const sm = sm0 + h * F::BUF;
+  auto sync = [h] { asm volatile("bar.sync %0, %1;" ::"r"(1 + h), "n"(F::T) : "memory"); };
+  float2* col = I.S + (size_t)(kx == F::L ? 0 : kx) * I.lds;
+  pdl_wait_prerequisites();
+  float2 x[F::E];
+  if (kx == 0 || kx == F::L) {
+    const float* c1 = reinterpret_cast<const float*>(col) + (kx == 0 ? 0 : 1);
+    static_for<0, F::E>([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const int j = t + F::T * q;
+      x[q] = make_float2(j < N ? c1[2 * j] : 0.f, 0.f);
+    });
+  } else {
+    static_for<0, F::E>([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const int j = t + F::T * q;
+      x[q] = j < N ? col[j] : make_float2(0.f, 0.f);
+    });
+  }
+  // odd half: frequencies m + 1/2 of the length-L transform
+  const float2* tw1 = h ? I.tw1h : I.tw1;
+  F::fwd(x, sm, t, tw1, h, I.tw2, sync);
+  // the symbol at y frequency 2 m + h, stored for 0 .. N' (it is even)
+  const float* lam = I.lnat + (size_t)kx * (F::L + 1);
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int k2 = 2 * (t + F::T * q) + h;
+    x[q] = cscale(x[q], __ldg(&lam[q < F::E / 2 ? k2 : 2 * F::L - k2]));
+  });
+  F::inv(x, sm, t, tw1, h, I.tw2, sync);
+  // even + odd half: the odd threads hand over the rows of
+  // q < E/2, the even threads the others, and each finishes its own rows
+  constexpr int HE = F::E / 2;
+  static_for<0, HE>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    sm[t + F::T * q] = h ? x[q] : x[q + HE];
+  });
+  __syncthreads();
+  const float2* other = sm0 + (h ^ 1) * F::BUF + t;
+  static_for<0, HE>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int j = t + F::T * (h ? q + HE : q);
+    const float2 y = cadd(h ? x[q + HE] : x[q], other[F::T * q]);
+    if (j < N) {
+      if (kx == 0) reinterpret_cast<float*>(col + j)[0] = y.x;
+      else if (kx == F::L) reinterpret_cast<float*>(col + j)[1] = y.x;
+      else col[j] = y;
+    }
+  });
+}
+
+// ---------------------------------------------------------------------------
+// Algorithm 1 on the bordered matrix: x = v' + i J v' (natural) -> vhat (its
+// factors Q and Q^H are the half-frequency shift of the first pair), then
+// y[q] = (H^-1 v)[k], k = t + T q: Re vhat[k] + Im vhat[N'-1-k] + the border
+// correction sum_p G[k, p] ybot[p], ybot[p] = Re vhat[N+p] + Im vhat[r-1-p];
+// for r > kBorderInline ybot of vector vec goes to YB, for border.cuh.
+template <int LOGL, typename Sync>
+__device__ __forceinline__ void gs_solve(float2* x, float* y, float2* sm, int t, int vec, const RegInst& I, Sync sync) {
+  using F = BlkFFT<LOGL>;
+  // skew-circulant factor lambda_s, then circulant factor lambda_c.  Rolled:
+  // one forward and one inverse transform body in the kernel.
+#pragma unroll 1
+  for (int round = 0; round < 2; ++round) {
+    const float2* lam = round == 0 ? I.lam_s : I.lam_c;
+    const float2* tw1 = round == 0 ? I.tw1h : I.tw1;
+    F::fwd(x, sm, t, tw1, round == 0, I.tw2, sync);
+    static_for<0, F::E>([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      x[q] = cmul(x[q], __ldg(&lam[t + F::T * q]));
+    });
+    F::inv(x, sm, t, tw1, round == 0, I.tw2, sync);
+  }
+  static_for<0, F::E>([&](auto qc) { sm[t + F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
+  sync();
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    y[q] = x[q].x + sm[F::L - 1 - (t + F::T * q)].y;
+  });
+  const int N = I.N, r = I.r;
+  if (r > kBorderInline) {
+    if (vec < N)
+      for (int p = t; p < r; p += F::T) I.YB[(size_t)p * I.ld + vec] = sm[N + p].x + sm[r - 1 - p].y;
+    return;
+  }
+#pragma unroll 1
+  for (int p = 0; p < r; ++p) {
+    const float yb = sm[N + p].x + sm[r - 1 - p].y;
+    const float* Gp = I.G + (size_t)p * N;
+    static_for<0, F::E>([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const int k = t + F::T * q;
+      if (k < N) y[q] += __ldg(Gp + k) * yb;
+    });
+  }
+}
+
+// ---------------------------------------------------------------------------
+// DENSE: the dense-inverse form stops after B^n, which it writes to W (FP32)
+// and, split into BF16 pairs, to Bh / Bl (the first sweep GEMM's A operand).
+// Else W receives the x sweep by columns, W[k * ld + row].
+template <int LOGL, bool DENSE>
+__global__ void __launch_bounds__(BlkFFT<LOGL>::T, DENSE ? Cfg<LOGL>::kDenseBlocks : Cfg<LOGL>::kGsBlocks)
+kb_rows_solve(const __grid_constant__ RegBatch B) {
+  using F = BlkFFT<LOGL>;
+  using C = Cfg<LOGL>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* sm = reinterpret_cast<float2*>(smem_raw);
+  pdl_allow_dependents();
+  const RegInst& I = B.in[blockIdx.y];
+  const int N = I.N, t = threadIdx.x;
+  const int rank = blockIdx.x % C::V, row0 = blockIdx.x - rank, row = blockIdx.x;
+  if (row0 >= N) return;   // the whole cluster
+  const bool valid = row < N;
+  const size_t rbase = (size_t)(valid ? row : 0) * I.ld;
+  auto sync = [] { __syncthreads(); };
+  cluster_arrive_relaxed();   // peers may be written once every block runs
+  // the rows the B^n epilogue reads into L2 under the convolution's tail
+  // (written in the previous step; a prefetch cannot make a load see older data)
+  if (valid) {
+    for (int c0 = 32 * t; c0 < N; c0 += 32 * F::T) {
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(I.C_hi + rbase + c0));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(I.C_lo + rbase + c0));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(I.u_hi + rbase + c0));
+    }
+  }
+  pdl_wait_prerequisites();
+  if constexpr (DENSE) {
+    // zero the sweep GEMM's counters for the GEMM that follows
+    if (blockIdx.x == 0 && I.dep)
+      for (int i = t; i < I.ndep; i += F::T) I.dep[i] = 0;
+  }
+  float2 x[F::E];
+  {
+    // frequencies rank L/V .. of the cluster's V rows, handed to their rows
+    const int vv = t % C::V, s0 = t / C::V;
+    const bool ok = row0 + vv < N;
+    const float2* col = I.S + (size_t)(rank * C::SEG + s0) * I.lds + row0 + (ok ? vv : 0);
+    static_for<0, F::E>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      x[i] = ok ? ld_stream(col + (size_t)(F::T / C::V * i) * I.lds) : make_float2(0.f, 0.f);
+    });
+    cluster_wait();
+    const unsigned dst = peer(sm + rank * C::SEG + s0, vv);
+    static_for<0, F::E>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      st_peer(dst + (unsigned)(F::T / C::V * i * sizeof(float2)), x[i]);
+    });
+  }
+  cluster_sync();
+  // half spectrum X[k] -> Z[k] = E + i O, the spectrum of z[n] = x[2n] + i x[2n+1]
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int k = t + F::T * q;
+    const float2 X = sm[k], Xc = cconj(sm[(F::L - k) & (F::L - 1)]);
+    const float2 Ev = cscale(cadd(X, Xc), 0.5f);
+    const float2 Ov = cscale(cmulc(csub(X, Xc), __ldg(&I.tw[k])), 0.5f);
+    x[q] = (q == 0 && t == 0) ? make_float2(0.5f * (X.x + X.y), 0.5f * (X.x - X.y)) : cadd(Ev, cmul_pi(Ov));
+  });
+  sync();
+  F::inv(x, sm, t, I.tw1, false, I.tw2, sync);
+  // x[q], q < E/2, now holds the convolution at 2n, 2n + 1, n = t + T q.
+  // Wave step: B = C + tau^2 (g(u) + f), n = 0: tau phi2 + (C + tau^2 (g + f))/2,
+  // with C <- C + conv; diffusion: B = C + conv/2 + tau (g(u~) + f) - d,
+  // u~ = u + d/2.  The equation is uniform over the launch.
+  const float tau = I.tau, tau2 = I.tau2;
+  auto bn = [&](auto diff_c) {
+    constexpr bool DIFF = decltype(diff_c)::value;
+    constexpr int HE = F::E / 2, GR = HE < 8 ? HE : 8;
+    static_for<0, HE / GR>([&](auto gc) {
+      constexpr int q0 = decltype(gc)::value * GR;
+      float2 ch[GR], cl[GR], uv[GR];
+      [[maybe_unused]] float2 dv[GR];
+      static_for<0, GR>([&](auto jc) {
+        constexpr int j = decltype(jc)::value;
+        const int e = 2 * (t + F::T * (q0 + j));
+        const bool ok = valid && e < N;
+        const size_t at = ok ? rbase + e : 0;
+        const float2 z = make_float2(0.f, 0.f);
+        ch[j] = ok ? ld_stream(reinterpret_cast<const float2*>(I.C_hi + at)) : z;
+        cl[j] = ok ? ld_stream(reinterpret_cast<const float2*>(I.C_lo + at)) : z;
+        uv[j] = ok ? ld_stream(reinterpret_cast<const float2*>(I.u_hi + at)) : z;
+        if constexpr (DIFF) dv[j] = (ok && !I.first) ? ld_stream(reinterpret_cast<const float2*>(I.u_d + at)) : z;
+      });
+      static_for<0, GR>([&](auto jc) {
+        constexpr int j = decltype(jc)::value;
+        const int e0 = 2 * (t + F::T * (q0 + j));
+        float b[2] = {0.f, 0.f}, cn[2] = {0.f, 0.f}, cln[2] = {0.f, 0.f};
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int i = e0 + e;
+          if (valid && i < N) {
+            // C <- C + conv (two-sum into the double-float pair)
+            const float hi = e ? ch[j].y : ch[j].x, lo = e ? cl[j].y : cl[j].x;
+            const float cx = e ? x[q0 + j].y : x[q0 + j].x;
+            const float s = hi + cx;
+            const float bb = s - hi;
+            const float err = (hi - (s - bb)) + (cx - bb);
+            const float l2 = lo + err;
+            const float c = s + l2;
+            cn[e] = c;
+            cln[e] = l2 - (c - s);
+            const float u = e ? uv[j].y : uv[j].x;
+            if constexpr (!DIFF) {
+              float gs = g_of_b(I, u);
+              if (I.F) gs += I.fsc * I.F[rbase + i];
+              const float gg = tau2 * gs;
+              b[e] = I.first ? tau * I.phi2[rbase + i] + 0.5f * (c + gg) : c + gg;
+            } else {
+              const float d = e ? dv[j].y : dv[j].x;
+              float gs = g_of_b(I, u + 0.5f * d);
+              if (I.F) gs += I.fsc * I.F[rbase + i];
+              b[e] = (c + 0.5f * cx) + tau2 * gs - d;
+            }
+          }
+        }
+        // 8-byte stores, or the single element at N - 1 (the padding is never written)
+        if (valid && e0 + 1 < N) {
+          *reinterpret_cast<float2*>(I.C_hi + rbase + e0) = make_float2(cn[0], cn[1]);
+          *reinterpret_cast<float2*>(I.C_lo + rbase + e0) = make_float2(cln[0], cln[1]);
+        } else if (valid && e0 < N) {
+          I.C_hi[rbase + e0] = cn[0];
+          I.C_lo[rbase + e0] = cln[0];
+        }
+        if constexpr (DENSE) {
+          // B^n to W and its BF16 pairs (at e0 + 1 = N, the zero padding of
+          // the pairs, the split of 0 is stored)
+          if (valid && e0 < N) {
+            float* wr = I.W + rbase;
+            if (e0 + 1 < N) *reinterpret_cast<float2*>(wr + e0) = make_float2(b[0], b[1]);
+            else wr[e0] = b[0];
+            unsigned hi, lo;
+            split_bf16x2(b[0], b[1], &hi, &lo);
+            *reinterpret_cast<unsigned*>(I.Bh + (size_t)row * I.ldp + e0) = hi;
+            *reinterpret_cast<unsigned*>(I.Bl + (size_t)row * I.ldp + e0) = lo;
+          }
+        } else {
+          sm[t + F::T * (q0 + j)] = make_float2(b[0], b[1]);
+        }
+      });
+    });
+  };
+  if (I.eq == 1) bn(std::integral_constant<bool, true>{});
+  else bn(std::integral_constant<bool, false>{});
+  if constexpr (DENSE) {
+    return;
+  } else {
+    sync();
+    // B' + i J B'
+    const float* bf = reinterpret_cast<const float*>(sm);
+    static_for<0, F::E>([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const int k = t + F::T * q;
+      x[q] = make_float2(bf[k], bf[F::L - 1 - k]);
+    });
+    sync();
+    float y[F::E];
+    gs_solve<LOGL>(x, y, sm, t, row, I, sync);
+    cluster_join();   // every block of the cluster has read its buffer
+    float* smf = reinterpret_cast<float*>(sm);
+    static_for<0, C::V>([&](auto cc) {
+      constexpr int c = decltype(cc)::value;
+      const unsigned dst = peer(smf + rank * C::P1 + t, c);
+      static_for<0, C::QS>([&](auto jc) {
+        constexpr int j = decltype(jc)::value;
+        st_peer(dst + (unsigned)(F::T * j * sizeof(float)), y[c * C::QS + j]);
+      });
+    });
+    cluster_sync();
+    const int vv = t % C::V, s0 = t / C::V;
+    if (row0 + vv >= N) return;
+    const float* src = smf + vv * C::P1 + s0;
+#pragma unroll 4
+    for (int i = 0; i < F::E; ++i) {
+      const int k = rank * C::SEG + s0 + F::T / C::V * i;
+      if (k < N) I.W[(size_t)k * I.ld + row0 + vv] = src[F::T / C::V * i];
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Column i of W (row i of the array by columns): uhat = H^-1 W, then, on the
+// rows handed out over the cluster's V columns, the compensated leapfrog
+// d^{n+1} = d^n + uhat (d^1 = uhat), u^{n+1} = u^n + d^{n+1}, u = u_hi + u_lo.
+template <int LOGL>
+__global__ void __launch_bounds__(BlkFFT<LOGL>::T, Cfg<LOGL>::kColsBlocks)
+kb_cols_solve(const __grid_constant__ RegBatch B) {
+  using F = BlkFFT<LOGL>;
+  using C = Cfg<LOGL>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* sm = reinterpret_cast<float2*>(smem_raw);
+  float* smf = reinterpret_cast<float*>(smem_raw);
+  pdl_allow_dependents();
+  const RegInst& I = B.in[blockIdx.y];
+  const int N = I.N, t = threadIdx.x;
+  const int rank = blockIdx.x % C::V, i0 = blockIdx.x - rank, i = blockIdx.x;
+  if (i0 >= N) return;   // the whole cluster
+  const bool valid = i < N;
+  auto sync = [] { __syncthreads(); };
+  pdl_wait_prerequisites();
+  const float* w = I.W + (size_t)(valid ? i : 0) * I.ld;
+  float2 x[F::E];
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int k = t + F::T * q, k2 = F::L - 1 - k;
+    x[q] = make_float2((valid && k < N) ? w[k] : 0.f, (valid && k2 < N) ? w[k2] : 0.f);
+  });
+  float y[F::E];
+  gs_solve<LOGL>(x, y, sm, t, i, I, sync);
+  cluster_join();   // every block of the cluster has read its buffer
+  static_for<0, C::V>([&](auto cc) {
+    constexpr int c = decltype(cc)::value;
+    const unsigned dst = peer(smf + rank * C::P1 + t, c);
+    static_for<0, C::QS>([&](auto jc) {
+      constexpr int j = decltype(jc)::value;
+      st_peer(dst + (unsigned)(F::T * j * sizeof(float)), y[c * C::QS + j]);
+    });
+  });
+  cluster_sync();
+  const int vv = t % C::V, s0 = t / C::V;
+  if (i0 + vv >= N) return;
+  const float* src = smf + vv * C::P1 + s0;
+  if (I.r > kBorderInline) {
+    // uhat short of its border correction, by rows, for border.cuh
+    float* U = reinterpret_cast<float*>(I.S);
+#pragma unroll 4
+    for (int e = 0; e < F::E; ++e) {
+      const int j = rank * C::SEG + s0 + F::T / C::V * e;
+      if (j < N) U[(size_t)j * I.ld + i0 + vv] = src[F::T / C::V * e];
+    }
+    return;
+  }
+  const int first = I.first;
+#pragma unroll 1
+  for (int g = 0; g < F::E; g += 8) {
+    float hi[8], lo[8], dd[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int j = rank * C::SEG + s0 + F::T / C::V * (g + e);
+      const size_t at = (size_t)j * I.ld + i0 + vv;
+      hi[e] = j < N ? ld_stream(I.u_hi + at) : 0.f;
+      lo[e] = j < N ? ld_stream(I.u_lo + at) : 0.f;
+      dd[e] = (j < N && !first) ? ld_stream(I.u_d + at) : 0.f;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int j = rank * C::SEG + s0 + F::T / C::V * (g + e);
+      if (j >= N) continue;
+      const size_t at = (size_t)j * I.ld + i0 + vv;
+      const float d = dd[e] + src[F::T / C::V * (g + e)];
+      const float s = hi[e] + d;
+      const float bb = s - hi[e];
+      const float err = (hi[e] - (s - bb)) + (d - bb);
+      const float l2 = lo[e] + err;
+      const float h2 = s + l2;
+      I.u_hi[at] = h2;
+      I.u_lo[at] = l2 - (h2 - s);
+      I.u_d[at] = d;
+    }
+  }
+}
+
+template <int LOGL>
+cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense) {
+  using F = BlkFFT<LOGL>;
+  using C = Cfg<LOGL>;
+  static LaunchCache attr_done[kLauncherDevices];
+  const int dev = device_slot();
+  if (dev < 0) return cudaErrorInvalidDevice;
+  cudaError_t e;
+  if (!attr_done[dev].load(std::memory_order_acquire)) {
+    auto room = [](auto kernel, size_t bytes) {
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    if ((e = room(kb_rows_r2c<LOGL>, C::bytes)) || (e = room(kb_cols_conv<LOGL>, C::bytes_conv)) ||
+        (e = room(kb_rows_solve<LOGL, false>, C::bytes)) || (e = room(kb_rows_solve<LOGL, true>, C::bytes)) ||
+        (e = room(kb_cols_solve<LOGL>, C::bytes)))
+      return e;
+    attr_done[dev].store(1, std::memory_order_release);
+  }
+  // every kernel of the step is a programmatic dependent of the one before
+  // it; the row kernels run in clusters of V blocks
+  auto launch = [&](auto kernel, dim3 grid, int threads, size_t smem, bool cluster) {
+    cudaLaunchAttribute a[2];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    a[1].id = cudaLaunchAttributeClusterDimension;
+    a[1].val.clusterDim.x = C::V;
+    a[1].val.clusterDim.y = 1;
+    a[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = a;
+    cfg.numAttrs = cluster ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, b);
+  };
+  const dim3 rgrid((max_n + C::V - 1) / C::V * C::V, b.count);
+  if (ev) cudaEventRecord(ev[0], st);
+  if ((e = launch(kb_rows_r2c<LOGL>, rgrid, F::T, C::bytes, true))) return e;
+  if (ev) cudaEventRecord(ev[1], st);
+  if ((e = launch(kb_cols_conv<LOGL>, dim3(F::L + 1, b.count), 2 * F::T, C::bytes_conv, false))) return e;
+  if (ev) cudaEventRecord(ev[2], st);
+  if (dense) return launch(kb_rows_solve<LOGL, true>, rgrid, F::T, C::bytes, true);
+  const bool border = border::any(b);
+  if ((e = launch(kb_rows_solve<LOGL, false>, rgrid, F::T, C::bytes, true))) return e;
+  if (border && (e = border::launch<0>(b, max_n, st))) return e;
+  if (ev) cudaEventRecord(ev[3], st);
+  if ((e = launch(kb_cols_solve<LOGL>, rgrid, F::T, C::bytes, true))) return e;
+  if (border && (e = border::launch<1>(b, max_n, st))) return e;
+  if (ev) cudaEventRecord(ev[4], st);
+  return cudaSuccess;
+}
+
+}  // namespace blk
+}  // namespace sadi

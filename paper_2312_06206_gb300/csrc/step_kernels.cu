@@ -172,10 +172,11 @@ __device__ __forceinline__ T gs_out(const cx<T>* vh, int k, const Geom& g, const
 // With u2 (the diffusion step, FP64) the transformed rows are those of
 // u + beta (u - u2): the extrapolation u~ = u^n + (u^n - u^{n-1})/2; EXTRAP
 // selects that form at compile time (the other launches carry none of it).
+// ldu: row pitch of u and u2.
 template <typename T, bool EXTRAP = false>
 __global__ void __launch_bounds__(kThreads)
 k_rows_r2c(const T* __restrict__ u, cx<T>* __restrict__ S, Geom g, const cx<T>* __restrict__ stw,
-           const cx<T>* __restrict__ tw, int NR, const T* __restrict__ u2 = nullptr, T beta = T(0)) {
+           const cx<T>* __restrict__ tw, int NR, int ldu, const T* __restrict__ u2 = nullptr, T beta = T(0)) {
   pdl_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* buf = reinterpret_cast<cx<T>*>(smem_raw);
@@ -187,11 +188,11 @@ k_rows_r2c(const T* __restrict__ u, cx<T>* __restrict__ S, Geom g, const cx<T>* 
     const int v = t >> logNp, n = t & (Np - 1);
     T a = T(0), b = T(0);
     if (v < nrows) {
-      const T* row = u + (size_t)(row0 + v) * N;
+      const T* row = u + (size_t)(row0 + v) * ldu;
       if (2 * n < N) a = row[2 * n];
       if (2 * n + 1 < N) b = row[2 * n + 1];
       if constexpr (EXTRAP) {
-        const T* row2 = u2 + (size_t)(row0 + v) * N;
+        const T* row2 = u2 + (size_t)(row0 + v) * ldu;
         if (2 * n < N) a += beta * (a - row2[2 * n]);
         if (2 * n + 1 < N) b += beta * (b - row2[2 * n + 1]);
       }
@@ -438,13 +439,13 @@ k_rows_solve(const cx<T>* __restrict__ S, const T* __restrict__ u, const T* __re
           const size_t row = (size_t)(row0 + v);
           const cx<T>* e = buf + v * vs;
           if (k < N) {
-            const T b = rhs_at<T, DIFF>(rp, e, k, row * N + k, u, uaux, phi2, Ch, Cl);
-            W[row * N + k] = b;
+            const T b = rhs_at<T, DIFF>(rp, e, k, row * g.ld + k, u, uaux, phi2, Ch, Cl);
+            W[row * g.ld + k] = b;
             split_bf16(b, Bh + row * ldp + k, Bl + row * ldp + k);
           }
           if (k2 < N) {
-            const T b = rhs_at<T, DIFF>(rp, e, k2, row * N + k2, u, uaux, phi2, Ch, Cl);
-            W[row * N + k2] = b;
+            const T b = rhs_at<T, DIFF>(rp, e, k2, row * g.ld + k2, u, uaux, phi2, Ch, Cl);
+            W[row * g.ld + k2] = b;
             split_bf16(b, Bh + row * ldp + k2, Bl + row * ldp + k2);
           }
         }
@@ -462,8 +463,8 @@ k_rows_solve(const cx<T>* __restrict__ S, const T* __restrict__ u, const T* __re
         if (v < nrows) {
           const int row = row0 + v;
           const cx<T>* e = buf + v * vs;
-          if (k < N) ra[it] = rhs_at<T, DIFF>(rp, e, k, (size_t)row * N + k, u, uaux, phi2, Ch, Cl);
-          if (k2 < N) rb[it] = rhs_at<T, DIFF>(rp, e, k2, (size_t)row * N + k2, u, uaux, phi2, Ch, Cl);
+          if (k < N) ra[it] = rhs_at<T, DIFF>(rp, e, k, (size_t)row * g.ld + k, u, uaux, phi2, Ch, Cl);
+          if (k2 < N) rb[it] = rhs_at<T, DIFF>(rp, e, k2, (size_t)row * g.ld + k2, u, uaux, phi2, Ch, Cl);
         }
       }
     }
@@ -483,7 +484,7 @@ k_rows_solve(const cx<T>* __restrict__ S, const T* __restrict__ u, const T* __re
     gs_bottom<T>(buf, NR, vs, g);
     for (int t = threadIdx.x; t < nrows * N; t += blockDim.x) {
       const int v = t / N, k = t % N;
-      W[(size_t)(row0 + v) * N + k] = gs_out<T>(buf + v * vs, k, g, G);
+      W[(size_t)(row0 + v) * g.ld + k] = gs_out<T>(buf + v * vs, k, g, G);
     }
   }
 }
@@ -513,8 +514,8 @@ k_cols_solve(const T* __restrict__ W, const T* u_cur, T* u_prev, T* u_next, T* u
     const int i = i0 + c, k2 = Np - 1 - k;
     T a = T(0), b = T(0);
     if (i < N) {
-      if (k < N) a = W[(size_t)k * N + i];
-      if (k2 < N) b = W[(size_t)k2 * N + i];
+      if (k < N) a = W[(size_t)k * g.ld + i];
+      if (k2 < N) b = W[(size_t)k2 * g.ld + i];
     }
     buf[c * vs + sidx<T>(k)] = cmul(mkc(a, b), __ldg(&tw[k]));
   }
@@ -526,7 +527,7 @@ k_cols_solve(const T* __restrict__ W, const T* u_cur, T* u_prev, T* u_next, T* u
     const int i = i0 + c;
     if (i >= N) continue;
     const T uh = gs_out<T>(buf + c * vs, j, g, G);
-    const size_t idx = (size_t)j * N + i;
+    const size_t idx = (size_t)j * g.ld + i;
     const T uc = u_cur[idx];
     if (u_lo) {
       leapfrog_comp<T>(uc, uh, first, idx, u_prev, u_next, u_lo);
@@ -545,13 +546,13 @@ k_cols_solve(const T* __restrict__ W, const T* u_cur, T* u_prev, T* u_next, T* u
 // ---------------------------------------------------------------------------
 constexpr int kTT = 32;   // transpose tile
 
-__global__ void __launch_bounds__(kTT * 8) k_transpose_f32(const float* __restrict__ A, float* __restrict__ AT, int N) {
+__global__ void __launch_bounds__(kTT * 8) k_transpose_f32(const float* __restrict__ A, float* __restrict__ AT, int N, int ld) {
   pdl_entry();
   __shared__ float tile[kTT][kTT + 1];
   const int x0 = blockIdx.x * kTT, y0 = blockIdx.y * kTT;
   for (int r = threadIdx.y; r < kTT; r += 8) {
     const int y = y0 + r, x = x0 + threadIdx.x;
-    tile[r][threadIdx.x] = (y < N && x < N) ? A[(size_t)y * N + x] : 0.f;
+    tile[r][threadIdx.x] = (y < N && x < N) ? A[(size_t)y * ld + x] : 0.f;
   }
   __syncthreads();
   for (int r = threadIdx.y; r < kTT; r += 8) {
@@ -595,7 +596,7 @@ k_rows_gs(const T* __restrict__ WT, T* __restrict__ UT, Geom g, const cx<T>* __r
 // u^{n+1} from uhat^T by 32 x 32 tiles: the compensated leapfrog of
 // k_cols_solve, element (j, i) with uhat = UT[i][j]
 __global__ void __launch_bounds__(kTT * 8) k_transpose_leapfrog(const float* __restrict__ UT, float* u_cur,
-                                                                 float* d, float* u_lo, int N, int first) {
+                                                                 float* d, float* u_lo, int N, int ld, int first) {
   pdl_entry();
   __shared__ float tile[kTT][kTT + 1];
   const int i0 = blockIdx.x * kTT, j0 = blockIdx.y * kTT;
@@ -607,7 +608,7 @@ __global__ void __launch_bounds__(kTT * 8) k_transpose_leapfrog(const float* __r
   for (int r = threadIdx.y; r < kTT; r += 8) {
     const int j = j0 + r, i = i0 + threadIdx.x;
     if (j < N && i < N) {
-      const size_t idx = (size_t)j * N + i;
+      const size_t idx = (size_t)j * ld + i;
       leapfrog_comp<float>(u_cur[idx], tile[threadIdx.x][r], first, idx, d, u_cur, u_lo);
     }
   }
@@ -740,9 +741,9 @@ cudaError_t launch_step(const Geom& g, const StepTables<T>& tb, const Tiles& tl,
   const size_t rsm = NR * vbytes;
   unsigned short* const no_bf16 = nullptr;
   cudaError_t ce = extrap ? launch_dependent(k_rows_r2c<T, true>, rg, kt, rsm, st, u_cur, S, g, stw, tw, NR,
-                                             static_cast<const T*>(u_prev), T(0.5))
+                                             g.ld, static_cast<const T*>(u_prev), T(0.5))
                           : launch_dependent(k_rows_r2c<T>, rg, kt, rsm, st, static_cast<const T*>(Ch ? u_prev : u_cur),
-                                             S, g, stw, tw, NR, static_cast<const T*>(nullptr), T(0));
+                                             S, g, stw, tw, NR, g.ld, static_cast<const T*>(nullptr), T(0));
   if (ce != cudaSuccess) return ce;
   if (ev) cudaEventRecord(ev[1], st);
   ce = launch_cols_conv<T>(g, tb, CTc, S, st);
@@ -760,14 +761,14 @@ cudaError_t launch_step(const Geom& g, const StepTables<T>& tb, const Tiles& tl,
     float* WT = reinterpret_cast<float*>(S);
     float* UT = WT + (size_t)g.N * g.N;
     const dim3 tg((g.N + kTT - 1) / kTT, (g.N + kTT - 1) / kTT), tb8(kTT, 8);
-    ce = launch_dependent(k_transpose_f32, tg, tb8, 0, st, reinterpret_cast<const float*>(W), WT, g.N);
+    ce = launch_dependent(k_transpose_f32, tg, tb8, 0, st, reinterpret_cast<const float*>(W), WT, g.N, g.ld);
     if (ce == cudaSuccess)
       ce = launch_dependent(k_rows_gs<T>, rg, kt, rsm, st, reinterpret_cast<const T*>(WT), reinterpret_cast<T*>(UT), g,
                             stw, tw, ls, lc, tb.G, NR);
     if (ce == cudaSuccess)
       ce = launch_dependent(k_transpose_leapfrog, tg, tb8, 0, st, static_cast<const float*>(UT),
                             reinterpret_cast<float*>(const_cast<T*>(u_cur)), reinterpret_cast<float*>(u_prev),
-                            reinterpret_cast<float*>(u_lo), g.N, rp.first);
+                            reinterpret_cast<float*>(u_lo), g.N, g.ld, rp.first);
   } else {
     ce = launch_dependent(k_cols_solve<T>, dim3((g.N + CTs - 1) / CTs), kt, CTs * vbytes, st,
                           static_cast<const T*>(W), u_cur, u_prev, u_next, u_lo, g, rp.first, stw, tw, ls, lc, tb.G,
@@ -792,8 +793,8 @@ template cudaError_t launch_step<double>(const Geom&, const StepTables<double>&,
                                          cudaStream_t, cudaEvent_t*, float*, float*);
 
 template <typename T>
-cudaError_t launch_remainder(const Geom& g, const StepTables<T>& tb, const Tiles& tl, const T* u, void* Sv, float* Ch,
-                             float* Cl, cudaStream_t st) {
+cudaError_t launch_remainder(const Geom& g, const StepTables<T>& tb, const Tiles& tl, const T* u, int ldu, void* Sv,
+                             float* Ch, float* Cl, cudaStream_t st) {
   const cx<T>* stw = reinterpret_cast<const cx<T>*>(tb.stw);
   const cx<T>* tw = reinterpret_cast<const cx<T>*>(tb.tw);
   cx<T>* S = reinterpret_cast<cx<T>*>(Sv);
@@ -801,16 +802,16 @@ cudaError_t launch_remainder(const Geom& g, const StepTables<T>& tb, const Tiles
   if (!tiles_valid<T>(g, tl)) return cudaErrorInvalidConfiguration;
   const int NR = tl.rows, CTc = tl.conv_cols;
   const int rblocks = (g.N + NR - 1) / NR;
-  k_rows_r2c<T><<<rblocks, kThreads, NR * vbytes, st>>>(u, S, g, stw, tw, NR);
+  k_rows_r2c<T><<<rblocks, kThreads, NR * vbytes, st>>>(u, S, g, stw, tw, NR, ldu);
   cudaError_t ce = launch_cols_conv<T>(g, tb, CTc, S, st);
   if (ce != cudaSuccess) return ce;
   k_rows_remainder<T><<<rblocks, kThreads, NR * vbytes, st>>>(S, g, stw, tw, NR, Ch, Cl);
   return cudaGetLastError();
 }
-template cudaError_t launch_remainder<float>(const Geom&, const StepTables<float>&, const Tiles&, const float*, void*,
-                                             float*, float*, cudaStream_t);
+template cudaError_t launch_remainder<float>(const Geom&, const StepTables<float>&, const Tiles&, const float*, int,
+                                             void*, float*, float*, cudaStream_t);
 template cudaError_t launch_remainder<double>(const Geom&, const StepTables<double>&, const Tiles&, const double*,
-                                              void*, float*, float*, cudaStream_t);
+                                              int, void*, float*, float*, cudaStream_t);
 
 cudaError_t launch_dense_rows(const Geom& g, const StepTables<float>& tb, const Tiles& tl, const RhsParams& rp,
                               const float* u_cur, const float* d, const float* phi2, void* Sv, float* W,
@@ -830,7 +831,7 @@ cudaError_t launch_dense_rows(const Geom& g, const StepTables<float>& tb, const 
   // every kernel a programmatic dependent of the one before it
   const dim3 rg(rblocks);
   const size_t rsm = NR * vbytes;
-  cudaError_t ce = launch_dependent(k_rows_r2c<T>, rg, dim3(kThreads), rsm, st, d, S, g, stw, tw, NR,
+  cudaError_t ce = launch_dependent(k_rows_r2c<T>, rg, dim3(kThreads), rsm, st, d, S, g, stw, tw, NR, g.ld,
                                     static_cast<const T*>(nullptr), T(0));
   if (ce != cudaSuccess) return ce;
   if (ev) cudaEventRecord(ev[1], st);

@@ -1,4 +1,4 @@
-// step_reg.cu -- dispatch of the register-FFT step path by FFT length.
+// step_reg.cu -- dispatch of the register-FFT step paths by FFT length.
 #include "../../include/sadi.h"
 #include "sadi_internal.h"
 
@@ -7,13 +7,14 @@ namespace regk {
 template <int LOGL>
 cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense);
 }  // namespace regk
+namespace blk {
+template <int LOGL>
+cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense);
+}  // namespace blk
 
-// both FP32 forms up to N' = 1024; the dense-inverse form's FFT part (its
-// sweeps are GEMMs) up to N' = 2048
+// both FP32 forms at every FFT length
 bool reg_path_supported(int logNp, int prec) {
-  if (prec == SADI_PREC_FP32) return logNp >= 3 && logNp <= 10;
-  if (prec == SADI_PREC_FP32_DENSE) return logNp >= 3 && logNp <= 11;
-  return false;
+  return (prec == SADI_PREC_FP32 || prec == SADI_PREC_FP32_DENSE) && logNp >= 3 && logNp <= 13;
 }
 
 cudaError_t launch_step_reg(const RegBatch& b, int logNp, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense) {
@@ -27,7 +28,9 @@ cudaError_t launch_step_reg(const RegBatch& b, int logNp, int max_n, cudaStream_
     case 8: return regk::launch_reg_impl<8>(b, max_n, st, ev, dense);
     case 9: return regk::launch_reg_impl<9>(b, max_n, st, ev, dense);
     case 10: return regk::launch_reg_impl<10>(b, max_n, st, ev, dense);
-    case 11: return regk::launch_reg_impl<11>(b, max_n, st, ev, dense);
+    case 11: return blk::launch_blk_impl<11>(b, max_n, st, ev, dense);
+    case 12: return blk::launch_blk_impl<12>(b, max_n, st, ev, dense);
+    case 13: return blk::launch_blk_impl<13>(b, max_n, st, ev, dense);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -1,6 +1,6 @@
 // step_reg.cuh -- the S-ADI step (Sec. 3, eq. "ADI scheme equivalent") for
-// FFT lengths N' <= 1024 (both FP32 forms) and N' = 2048 (the dense-inverse
-// form's FFT part) with the register-resident two-level FFT of regfft.cuh.
+// FFT lengths N' <= 1024 (both FP32 forms) with the register-resident
+// two-level FFT of regfft.cuh (longer lengths: step_blk.cuh).
 // Same four kernels and the same mathematics as step_kernels.cu:
 //   kr_rows_r2c    rows of the increment d^n = u^n - u^{n-1} -> half spectrum
 //                  along x (natural slots)
@@ -61,9 +61,8 @@ struct RowCfg {
   static constexpr size_t bytes_r2c = (size_t)VB * SMV * sizeof(float2) + tw_bytes;
   static constexpr size_t bytes_solve = (size_t)VB * SMV * sizeof(float2) + tw_bytes;
   // resident blocks per SM promised to the compiler (its register budget):
-  // four narrow blocks (two at N' = 2048, whose 64 elements per lane need
-  // the full 255 registers), or one wide block of up to 2048 threads
-  static constexpr int kMinBlocks = BLOCK >= 512 ? 1 : (LOGL >= 11 ? 2 : 4);
+  // four narrow blocks, or one wide block of up to 2048 threads
+  static constexpr int kMinBlocks = BLOCK >= 512 ? 1 : 4;
 };
 // The convolution kernel: vectors owned by warps (as in the row kernels), CT
 // per block; the FFT buffers and the staged table tw1 (the symbol rows are
@@ -81,7 +80,7 @@ struct ConvCfg {
   // the half-angle twiddles tw[0 .. L) are staged too when the shared memory
   // still admits the block count of the launch bounds
   static constexpr size_t bytes_base = (size_t)CT * SMV * sizeof(float2) + (size_t)F::L * sizeof(float2);
-  static constexpr int kBlocksPerSm = BLOCK >= 256 || LOGL >= 11 ? 2 : 4;
+  static constexpr int kBlocksPerSm = BLOCK >= 256 ? 2 : 4;
   static constexpr bool STAGE_TW =
       kBlocksPerSm * (bytes_base + F::L * sizeof(float2) + 1024) <= (size_t)228 * 1024;
   static constexpr size_t bytes = bytes_base + (STAGE_TW ? F::L * sizeof(float2) : 0);
@@ -289,7 +288,7 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   F::template fwd<true>(x, sm, t, s_tw1);
   store_freq<LOGL>(x, sm, t);
   __syncthreads();
-  // the spectrum is slot-major, S[k * N + row]: the block writes slot by slot,
+  // the spectrum is slot-major, S[k * lds + row]: the block writes slot by slot,
   // its rows fastest (runs of VB rows), reading every vector's buffer
   const float2* base = reinterpret_cast<const float2*>(smem_raw);
   const int row0 = blockIdx.x * C::VB;
@@ -308,12 +307,12 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
     const float2 Zc = cconj(Zp);
     const float2 Ev = cscale(cadd(Z, Zc), 0.5f);
     const float2 Ov = cscale(cmul_mi(csub(Z, Zc)), 0.5f);
-    col[(size_t)k * N] = (k == 0) ? make_float2(Ev.x + Ov.x, Ev.x - Ov.x) : cadd(Ev, cmul(s_tw[k], Ov));
+    col[(size_t)k * I.lds] = (k == 0) ? make_float2(Ev.x + Ov.x, Ev.x - Ov.x) : cadd(Ev, cmul(s_tw[k], Ov));
     if (kp != k) {
       const float2 Zc2 = cconj(Z);
       const float2 Ev2 = cscale(cadd(Zp, Zc2), 0.5f);
       const float2 Ov2 = cscale(cmul_mi(csub(Zp, Zc2)), 0.5f);
-      col[(size_t)kp * N] = cadd(Ev2, cmul(s_tw[kp], Ov2));
+      col[(size_t)kp * I.lds] = cadd(Ev2, cmul(s_tw[kp], Ov2));
     }
   }
 }
@@ -347,7 +346,7 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
   auto kx_of = [&](int it) { return (it == 0 || it > Np) ? 0 : (it == 1 ? Np : it - 1); };
   for (int e = threadIdx.x; e < F::L; e += BLOCK) cp_async8(&s_tw1[e], I.tw1 + e, true);
   // each item's column, rows 0 .. N-1 (zero-filled to L), once, into the
-  // buffer of its even-half vector: the spectrum is slot-major (S[k * N + j]),
+  // buffer of its even-half vector: the spectrum is slot-major (S[k * lds + j]),
   // so a column is contiguous; thread -> (item, row) with the rows fastest
   pdl_wait_prerequisites();
   constexpr int NI = C::CT / 2;
@@ -355,7 +354,7 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
     const int j = e % F::L, ci = e / F::L, it = item_of(2 * ci);
     float2* dst = reinterpret_cast<float2*>(smem_raw) + 2 * ci * C::SMV + pad32(j);
     const bool ok = it <= Np && j < N;
-    cp_async8(dst, I.S + (size_t)(ok ? slot_of(it) : 0) * N + (ok ? j : 0), ok);
+    cp_async8(dst, I.S + (size_t)(ok ? slot_of(it) : 0) * I.lds + (ok ? j : 0), ok);
   }
   cp_async_commit();
   cp_async_wait_all();
@@ -402,7 +401,7 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
     const int it = item_of(2 * i);
     if (it > Np || it == 1) continue;
     const float2* se = base + (2 * i) * C::SMV;
-    float2* col = I.S + (size_t)slot_of(it) * N;
+    float2* col = I.S + (size_t)slot_of(it) * I.lds;
     for (int j = threadIdx.x; j < N; j += BLOCK) {
       const float2 w = twh[j];
       const float2 y = cadd(se[pad32(j)], cmulc(se[C::SMV + pad32(j)], w));
@@ -458,7 +457,7 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
     if (blockIdx.x == 0 && I.dep)
       for (int i = threadIdx.x; i < I.ndep; i += BLOCK) I.dep[i] = 0;
   }
-  // stage the block's spectrum rows from the slot-major spectrum S[k * N + row]
+  // stage the block's spectrum rows from the slot-major spectrum S[k * lds + row]
   // (slot by slot, rows fastest: runs of VB rows); u^n, and phi2 on the
   // first step, are read in the B^n epilogue together with the remainder
   {
@@ -470,7 +469,7 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
     const float2* col = I.S + (ok ? row0 + vv : 0);
     float2* dst = base + vv * C::SMV;
     for (int k = threadIdx.x / C::VB; k < F::L; k += BLOCK / C::VB)
-      cp_async8(&dst[pad32(k)], col + (ok ? (size_t)k * N : 0), ok);
+      cp_async8(&dst[pad32(k)], col + (ok ? (size_t)k * I.lds : 0), ok);
   }
   cp_async_commit();
   cp_async_wait_all();
@@ -733,21 +732,11 @@ inline bool fewer_waves(int shape, int count, int max_n, int narrow_rows, int wi
   return (wb + sms * ow - 1) / (sms * ow) < (nb + sms * on - 1) / (sms * on);
 }
 
-// FFT lengths of the register path: both FP32 forms up to 2^kRegMaxLogGS, the
-// dense-inverse form's FFT part (no GS sweeps) up to 2^kRegMaxLogDense.  At
-// N' = 2048 the GS sweep kernels would hold 64 elements per lane at the full
-// register budget, 2 blocks per SM, and measured slower than the
-// shared-memory engine's; the dense form's three kernels measured faster.
-constexpr int kRegMaxLogGS = 10;
-constexpr int kRegMaxLogDense = 11;
+constexpr int kRegMaxLog = kBlkMinLog - 1;   // longer vectors: step_blk.cuh
 
 template <int LOGL>
 cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense) {
-  static_assert(LOGL <= kRegMaxLogDense, "register path FFT length");
-  // the GS form's kernels (and the wide row blocks, N' = 1024 only) exist at
-  // the lengths that use them
-  constexpr bool kGS = LOGL <= kRegMaxLogGS;
-  if (!kGS && !dense) return cudaErrorInvalidValue;
+  static_assert(LOGL <= kRegMaxLog, "register path FFT length");
   using RC = RowCfg<LOGL, kRowBlock>;
   using CC = ColCfg<LOGL, kColBlock>;
   using VC = ConvCfg<LOGL, kConvBlock>;
@@ -791,13 +780,11 @@ cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
         (e = cudaFuncSetAttribute(kr_cols_conv<LOGL, kConvBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)VC::bytes)))
       return e;
-    if constexpr (kGS) {
-      if ((e = cudaFuncSetAttribute(kr_rows_solve<LOGL, kRowBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)RC::bytes_solve)) ||
-          (e = cudaFuncSetAttribute(kr_cols_solve<LOGL, kColBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)CC::bytes_solve)))
-        return e;
-    }
+    if ((e = cudaFuncSetAttribute(kr_rows_solve<LOGL, kRowBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)RC::bytes_solve)) ||
+        (e = cudaFuncSetAttribute(kr_cols_solve<LOGL, kColBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)CC::bytes_solve)))
+      return e;
     attr_done[dev].store(1, std::memory_order_release);
   }
   const dim3 rgrid((max_n + RC::VB - 1) / RC::VB, b.count);
@@ -842,18 +829,16 @@ cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
     }
     return launch(kr_rows_solve<LOGL, kRowBlock, true>, rgrid, kRowBlock, RC::bytes_solve);
   }
-  if constexpr (kGS) {
-    if constexpr (LOGL == 10) {
-      if (wide[1]) e = launch(kr_rows_solve<LOGL, kRowBlockWide>, wgrid, kRowBlockWide, RW::bytes_solve);
-      else e = launch(kr_rows_solve<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_solve);
-    } else {
-      e = launch(kr_rows_solve<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_solve);
-    }
-    if (e != cudaSuccess) return e;
-    if (ev) cudaEventRecord(ev[3], st);
-    if ((e = launch(kr_cols_solve<LOGL, kColBlock>, sgrid, kColBlock, CC::bytes_solve))) return e;
-    if (ev) cudaEventRecord(ev[4], st);
+  if constexpr (LOGL == 10) {
+    if (wide[1]) e = launch(kr_rows_solve<LOGL, kRowBlockWide>, wgrid, kRowBlockWide, RW::bytes_solve);
+    else e = launch(kr_rows_solve<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_solve);
+  } else {
+    e = launch(kr_rows_solve<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_solve);
   }
+  if (e != cudaSuccess) return e;
+  if (ev) cudaEventRecord(ev[3], st);
+  if ((e = launch(kr_cols_solve<LOGL, kColBlock>, sgrid, kColBlock, CC::bytes_solve))) return e;
+  if (ev) cudaEventRecord(ev[4], st);
   return cudaSuccess;
 }
 

@@ -1,0 +1,103 @@
+"""The block-FFT path of the FP32 forms (FFT lengths 2048 .. 8192) against the
+shared-memory engine (explicit tiles) and the FP64 path, at the sizes where its
+clusters of eight rows, its slot runs and its border correction change: the
+smallest N of a length, N one above and below a multiple of eight, border ranks
+32 (added inside the sweep kernels), 33 and 1023 (one product per sweep), and
+N = N' (no border).
+
+Tolerances: both engines compute the same FP32 transforms in different orders.
+One transform of length L carries a relative error of about eps log2 L
+(6e-8 x 13 < 1e-6) and the increment it yields is at most tau ||u_t|| / ||u|| <
+1e-1 of the field per step here, so three steps agree to 1e-6 of the largest
+value; the FP32 forms' bound against FP64 is 1e-5."""
+import numpy as np
+import pytest
+
+from paper_2312_06206_gb300 import workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def S():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_06206_gb300 import build
+    build.build()
+    from paper_2312_06206_gb300 import sadi
+    return sadi
+
+
+def _run(S, N, prec, equation, tiles=False, g=3):
+    tau = 1e-3 if equation == "wave" else 3e-6
+    phi1 = WL.gaussian_bumps(N, 6, 3000 + N)
+    phi2 = 0.1 * WL.gaussian_bumps(N, 3, 3100 + N) if equation == "wave" else None
+    with S.Sadi(N, 1.4, 0.9, tau, equation=equation) as s:
+        s.sadi_set_nonlinearity(-1.0, -0.5, 0.25)
+        s.set_options(g, prec)
+        if tiles:
+            s.sadi_set_tiles(*s.sadi_get_tiles())
+        s.set_initial(phi1, phi2)
+        s.step(3)
+        return s.get()[0]
+
+
+@pytest.mark.parametrize("N", [1025, 2015, 2016, 2041, 2048, 4089, 4095, 4096])
+@pytest.mark.parametrize("equation", ["wave", "diffusion"])
+@pytest.mark.parametrize("prec_name", ["SADI_PREC_FP32", "SADI_PREC_FP32_DENSE"])
+def test_block_path_against_shared_memory_engine(S, N, equation, prec_name):
+    prec = getattr(S, prec_name)
+    u = _run(S, N, prec, equation)
+    v = _run(S, N, prec, equation, tiles=True)
+    assert not np.array_equal(u, v)          # two engines, not one
+    assert np.abs(u - v).max() <= 1e-6 * np.abs(v).max()
+    if N in (1025, 2015, 2048):
+        w = _run(S, N, S.SADI_PREC_FP64, equation)
+        assert np.abs(u - w).max() <= 1e-5 * np.abs(w).max()
+
+
+def test_block_path_batch_of_uneven_border_ranks(S):
+    # one launch per kernel for members of N' = 2048 with r = 1, 33 and 0;
+    # bitwise what each gives alone
+    Ns = [2047, 2015, 2048]
+    phis = [WL.gaussian_bumps(N, 4, 3200 + N) for N in Ns]
+
+    def make():
+        out = []
+        for N, p in zip(Ns, phis):
+            s = S.Sadi(N, 1.5, 1.0, 1e-3)
+            s.set_options(1, S.SADI_PREC_FP32)
+            s.set_initial(p)
+            out.append(s)
+        return out
+    alone, batch = make(), make()
+    for s in alone:
+        s.step(3)
+    S.sadi_batch_step(batch, 3)
+    for a, b in zip(alone, batch):
+        assert np.array_equal(a.get()[0], b.get()[0])
+        a.close()
+        b.close()
+
+
+def test_tiles_move_a_running_context_between_the_engines(S):
+    # both engines keep the state in one layout: an FP32 context may change
+    # engine between steps
+    N = 1100
+    phi1 = WL.gaussian_bumps(N, 4, 3300)
+    us = []
+    for switch in (False, True):
+        with S.Sadi(N, 1.5, 1.0, 1e-3) as s:
+            s.set_options(1, S.SADI_PREC_FP32)
+            s.set_initial(phi1)
+            s.step(2)
+            if switch:
+                s.sadi_set_tiles(*s.sadi_get_tiles())
+            s.step(2)
+            if switch:
+                s.sadi_set_tiles(0, 0, 0)
+            s.step(1)
+            us.append(s.get()[0])
+    assert not np.array_equal(us[0], us[1])
+    assert np.abs(us[0] - us[1]).max() <= 1e-6 * np.abs(us[0]).max()
