@@ -74,6 +74,18 @@ __device__ __forceinline__ void idft(float2* x) {
 template <int LOGL>
 struct Radix;
 template <>
+struct Radix<8> {
+  static constexpr int R1 = 8, R2 = 4, R3 = 8;
+};
+template <>
+struct Radix<9> {
+  static constexpr int R1 = 8, R2 = 8, R3 = 8;
+};
+template <>
+struct Radix<10> {
+  static constexpr int R1 = 16, R2 = 8, R3 = 8;
+};
+template <>
 struct Radix<11> {
   static constexpr int R1 = 16, R2 = 8, R3 = 16;
 };

@@ -26,13 +26,12 @@ constexpr int kTile = 64, kK = 16, kThreads = 256;
 template <int MODE>
 __global__ void __launch_bounds__(kThreads) k_border(const __grid_constant__ RegBatch B) {
   __shared__ __align__(16) float sp[2][kK][kTile], sq[2][kK][kTile];
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const RegInst& I = B.in[blockIdx.z];
   const int N = I.N, r = I.r;
   const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
   if (r <= kBorderInline || m0 >= N || n0 >= N) return;
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_entry();
   const float* P = MODE == 2 ? I.YB : I.G;
   const float* Q = MODE == 2 ? I.G : I.YB;
   const int ldp = MODE == 2 ? I.ld : N, ldq = MODE == 2 ? N : I.ld;

@@ -264,7 +264,7 @@ sadi_status sadi_autotune(sadi_ctx** ctxs, int count, int g, int flags) {
       if ((st = time_group(grp, 5, &ms)) != SADI_OK) return st;
       // the shared-memory engine's decompositions beside the register path,
       // where the GS form may run on either (explicit tiles)
-      if (prec == SADI_PREC_FP32 && logNp >= kBlkMinLog) {
+      if (prec == SADI_PREC_FP32 && logNp >= kTilesMinLog) {
         // coordinate descent over the shared-memory engine's decomposition;
         // the column convolution may also run as three passes (kConvThreePass)
         Tiles t = grp[0]->tiles32;

@@ -56,7 +56,7 @@ void free_all(sadi_ctx* c) {
   for (void* p : ptrs)
     if (p) cudaFree(p);
   conv3_free(&c->c3);
-  void* dense[] = {c->Eh, c->El, c->Bh, c->Bl, c->WTh, c->WTl, c->tcerr, c->tcdep, c->Chi, c->Clo, c->wd, c->Fconv};
+  void* dense[] = {c->Eh, c->El, c->Bh, c->Bl, c->WTh, c->WTl, c->tcerr, c->tcdep, c->Chi, c->Clo, c->wd, c->Fconv, c->dF, c->dT, c->dE};
   for (void* p : dense)
     if (p) cudaFree(p);
   for (auto& a : c->ev_pool)
@@ -96,9 +96,9 @@ int log2i(int v) {
   return l;
 }
 
-// rows per slot of the register paths' spectrum (RegInst::lds): from N' = 2048
-// on a multiple of 8, so that the 8-row runs of a cluster stay aligned
-int slot_rows(const sadi::Geom& g) { return g.logNp < kBlkMinLog ? g.N : (g.N + 7) / 8 * 8; }
+// rows per slot of the block path's spectrum (RegInst::lds): a multiple of 8,
+// so that the 8-row runs of a cluster stay aligned
+int slot_rows(int N) { return (N + 7) / 8 * 8; }
 
 size_t esize(int prec) { return prec == SADI_PREC_FP64 ? sizeof(double) : sizeof(float); }
 
@@ -107,7 +107,43 @@ size_t esize(int prec) { return prec == SADI_PREC_FP64 ? sizeof(double) : sizeof
 // has, select that engine from N' = 2048 on.
 bool wants_reg_path(const sadi_ctx* c) {
   if (!reg_path_supported(c->g.logNp, c->prec)) return false;
-  return !(c->tiles_explicit && c->g.logNp >= kBlkMinLog);
+  return !(c->tiles_explicit && c->g.logNp >= kTilesMinLog);
+}
+
+// Tables of the direct path for the context's precision (see dir_mode).
+// whether the direct path holds H^-1 as I + E: while the ADI factor I + s T is
+// within 1/2 of the identity in its diagonal, s a_0 <= 1/2 (a_0 < 2.01 for
+// every alpha; H^-1 = I + E then has no cancellation in B + B E)
+bool dir_ident(const sadi_ctx* c) { return 2.0 * c->s <= 0.5; }
+template <typename T>
+sadi_status build_direct(sadi_ctx* c, int mode) {
+  const size_t N = c->g.N;
+  cudaStream_t st = c->stream;
+  const size_t ebytes = N * c->g.ld * sizeof(T);
+  CK(cudaMalloc(&c->dE, ebytes), "cudaMalloc(direct path)");
+  CK(cudaMemsetAsync(c->dE, 0, ebytes, st), "direct path");
+  int stat = 1;
+  CK(run_dir_inverse<T>(c->a1, c->g.N, c->g.ld, c->s, dir_ident(c), static_cast<T*>(c->dE), &stat, st), "direct path inverse");
+  if (stat != 0) return fail(c, SADI_ENOTSPD, "Durbin recursion of the N x N generator broke down");
+  if (mode == 2) {   // FP64
+    CK(cudaMalloc(&c->dF, (2 * N + 2) * N * sizeof(double)), "cudaMalloc(direct path)");
+    CK(cudaMalloc(&c->dT, (N + 1) * N * sizeof(double)), "cudaMalloc(direct path)");
+    // kappa tau^2 h^-alpha (wave) or kappa tau h^-alpha (diffusion) is 2 s
+    CK(run_dir_tables(static_cast<double*>(c->dF), static_cast<double*>(c->dT), c->a2d, c->g.N, -2.0 * c->s, st),
+       "direct path tables");
+  }
+  return SADI_OK;
+}
+sadi_status setup_direct(sadi_ctx* c) {
+  for (void** p : {&c->dF, &c->dT, &c->dE}) {
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+  }
+  if (c->prec == SADI_PREC_FP32_DENSE) return SADI_OK;
+  const bool f64 = c->prec == SADI_PREC_FP64;
+  const int mode = dir_mode(c->g, f64);
+  if (mode == 0) return SADI_OK;
+  return f64 ? build_direct<double>(c, mode) : build_direct<float>(c, mode);
 }
 
 sadi_status alloc_state(sadi_ctx* c) {
@@ -139,9 +175,13 @@ sadi_status alloc_state(sadi_ctx* c) {
   // (the register paths' slots hold lds >= N rows each)
   const size_t ses = (c->prec != SADI_PREC_FP64 && c->g.Np <= 4096) ? sizeof(double) : es;
   const size_t sbytes = (size_t)c->g.N * c->g.Np * 2 * ses;
-  size_t rbytes = c->prec != SADI_PREC_FP64 ? (size_t)slot_rows(c->g) * c->g.Np * sizeof(float2) : 0;
+  size_t rbytes = c->prec != SADI_PREC_FP64 ? (size_t)slot_rows(c->g.N) * c->g.Np * sizeof(float2) : 0;
   // behind the slots: the bottom entries of the bordered solves
   if (c->prec == SADI_PREC_FP32 && c->g.r > kBorderInline) rbytes += (size_t)c->g.r * c->g.ld * sizeof(float);
+  // the direct path's V and Wm (their order in dir_inst)
+  const size_t dbytes = (3 * (size_t)c->g.N + 2) * c->g.ld * es;
+  if (c->prec != SADI_PREC_FP32_DENSE && dir_mode(c->g, c->prec == SADI_PREC_FP64) && dbytes > rbytes)
+    rbytes = dbytes;
   CK(cudaMalloc(&c->S, sbytes > rbytes ? sbytes : rbytes), "cudaMalloc(spectrum)");
   CK(cudaMalloc(&c->W, nn * es), "cudaMalloc(sweep)");
   if (c->g.ld != c->g.N) {
@@ -151,6 +191,8 @@ sadi_status alloc_state(sadi_ctx* c) {
     for (void* b : pbufs) CK(cudaMemsetAsync(b, 0, nn * es, c->stream), "zero state");
     CK(cudaStreamSynchronize(c->stream), "zero state");
   }
+  const sadi_status sd = setup_direct(c);
+  if (sd != SADI_OK) return sd;
   // FP32 forms whose explicit tiles select the three-pass column convolution:
   // its buffers and tables (kept once allocated)
   if (c->prec != SADI_PREC_FP64 && !c->reg_path && c->tiles32.conv_cols == kConvThreePass) {
@@ -283,8 +325,8 @@ sadi_status create_impl(int eq, int N, double alpha, double kappa, double tau, c
       {(void**)&c->G64, sizeof(double) * ((size_t)N * g.r + 1)},
       {(void**)&c->G32, sizeof(float) * ((size_t)N * g.r + 1)},
       {(void**)&c->stage, sizeof(double) * nn},
-      {(void**)&c->rtw1, sizeof(float2) * (2 * Np + kTw2)},
-      {(void**)&c->rlreg, sizeof(float) * reg_symbol_elems(g)},
+      {(void**)&c->rtw1, sizeof(float2) * (3 * Np + kTw2)},
+      {(void**)&c->rlreg, sizeof(float) * (reg_lreg_elems(g) + reg_lnat_elems(g))},
       {(void**)&c->rlamc, sizeof(float2) * Np},
       {(void**)&c->rlams, sizeof(float2) * Np},
       {(void**)&c->wd, sizeof(WdState)},
@@ -507,11 +549,13 @@ RhsParams rhs_of(const sadi_ctx* c, long long n) {
   rp.first = n == 0 ? 1 : 0;
   if (c->F_step) {
     rp.F = c->F_step;
+    rp.ldF = c->F_step == c->Fconv ? c->g.ld : c->g.N;
     rp.fsc = 1.0;
   } else if (c->F) {
     // the wave step samples f at t_n, the diffusion step at t_{n+1/2}
     const double t = ((double)n + (c->eq == 0 ? 0.0 : 0.5)) * c->tau;
     rp.F = c->F;
+    rp.ldF = c->g.ld;
     rp.fsc = std::cos(c->f_omega * t + c->f_phase);
   }
   rp.gc1 = c->gc[0];
@@ -522,21 +566,25 @@ RhsParams rhs_of(const sadi_ctx* c, long long n) {
 
 RegInst reg_inst(const sadi_ctx* c) {
   RegInst r{};
+  const int Np = c->g.Np;
   r.tw1 = c->rtw1;
-  r.tw2 = c->rtw1 + c->g.Np;
-  r.tw1h = r.tw2 + kTw2;
+  r.btw1 = r.tw1 + Np;
+  r.btw1h = r.btw1 + Np;
+  r.btw2 = r.btw1h + Np;
   r.tw = c->tw32;
   r.lam_s = c->rlams;
   r.lam_c = c->rlamc;
-  r.lreg = r.lnat = c->rlreg;
+  r.lreg = c->rlreg;
+  r.lnat = c->rlreg + reg_lreg_elems(c->g);
   r.G = c->G32;
   r.u_hi = static_cast<float*>(c->ubuf[0]);
   r.u_d = static_cast<float*>(c->ubuf[1]);
   r.u_lo = c->ulo;
   r.phi2 = static_cast<const float*>(c->phi2);
   r.S = static_cast<float2*>(c->S);
-  r.lds = slot_rows(c->g);
-  r.YB = reinterpret_cast<float*>(r.S + (size_t)r.lds * c->g.Np);
+  const bool blk = blk_path(c->g.logNp, c->prec == SADI_PREC_FP32_DENSE);
+  r.lds = blk ? slot_rows(c->g.N) : c->g.N;
+  r.YB = reinterpret_cast<float*>(r.S + (size_t)slot_rows(c->g.N) * c->g.Np);
   r.W = static_cast<float*>(c->W);
   r.N = c->g.N;
   r.ld = c->g.ld;
@@ -548,19 +596,70 @@ RegInst reg_inst(const sadi_ctx* c) {
   r.first = c->n == 0 ? 1 : 0;
   const RhsParams rp = rhs_of(c, c->n);
   r.F = static_cast<const float*>(rp.F);
+  r.ldF = rp.ldF;
   r.fsc = (float)rp.fsc;
   r.gc1 = (float)c->gc[0];
   r.gc3 = (float)c->gc[1];
   r.gcs = (float)c->gc[2];
   r.C_hi = c->Chi;
   r.C_lo = c->Clo;
-  r.Bh = c->Bh;
+  r.Bh = c->prec == SADI_PREC_FP32_DENSE ? c->Bh : nullptr;
   r.Bl = c->Bl;
   r.ldp = c->npad;
   r.dep = c->prec == SADI_PREC_FP32_DENSE ? c->tcdep : nullptr;
   r.ndep = c->npad / kTcBox + 1;
   return r;
 }
+
+// the direct path's view of a context at time level n; V and Wm in scratch
+template <typename T>
+DirInst<T> dir_inst(const sadi_ctx* c, long long n, void* scratch, T* Bm) {
+  DirInst<T> d{};
+  const RhsParams rp = rhs_of(c, n);
+  d.F = static_cast<const T*>(c->dF);
+  d.T_ = static_cast<const T*>(c->dT);
+  d.E = static_cast<const T*>(c->dE);
+  d.ident = dir_ident(c) ? 1 : 0;
+  d.N = c->g.N;
+  d.ld = c->g.ld;
+  d.V = static_cast<T*>(scratch);
+  d.Wm = d.V + (2 * (size_t)d.N + 2) * d.ld;
+  d.Bm = Bm;
+  d.phi2 = static_cast<const T*>(c->phi2);
+  d.src = static_cast<const T*>(rp.F);
+  d.fsc = (T)rp.fsc;
+  d.gkind = rp.g;
+  d.first = rp.first;
+  d.eq = rp.eq;
+  d.tau = (T)rp.tau;
+  d.tau2 = (T)rp.tau2;
+  d.gc1 = (T)rp.gc1;
+  d.gc3 = (T)rp.gc3;
+  d.gcs = (T)rp.gcs;
+  return d;
+}
+DirInst<float> dir_inst32(const sadi_ctx* c) {
+  DirInst<float> d = dir_inst<float>(c, c->n, c->S, static_cast<float*>(c->W));
+  d.u = d.next = static_cast<float*>(c->ubuf[0]);
+  d.aux = static_cast<float*>(c->ubuf[1]);
+  d.lo = c->ulo;
+  return d;
+}
+// one FP64 step from u_cur and u_prev to u_next
+cudaError_t dir_step64(const sadi_ctx* c, long long n, const double* u_cur, double* u_prev, double* u_next, void* S,
+                       double* W, cudaStream_t st, cudaEvent_t* ev) {
+  static thread_local DirBatch<double> b;
+  b.count = 1;
+  DirInst<double>& d = b.in[0];
+  d = dir_inst<double>(c, n, S, W);
+  d.u = d.x = u_cur;
+  d.aux = u_prev;
+  d.next = u_next;
+  d.x2 = u_prev;
+  d.beta = c->eq == 1 && !d.first ? 0.5 : 0.0;
+  return launch_dir_step(b, c->g.N, st, ev);
+}
+bool uses_direct64(const sadi_ctx* c) { return c->prec == SADI_PREC_FP64 && c->dF && !c->tiles64_explicit; }
 
 bool uses_reg_path(const sadi_ctx* c) { return c->prec == SADI_PREC_FP32 && c->reg_path; }
 bool is_dense(const sadi_ctx* c) { return c->prec == SADI_PREC_FP32_DENSE; }
@@ -574,9 +673,12 @@ sadi_status step_smem(sadi_ctx* c, cudaEvent_t* ev, cudaStream_t st) {
     void* ucur = c->ubuf[c->cur];
     void* uoth = c->ubuf[1 - c->cur];
     StepTables<double> tb{c->stw64, c->tw64, c->lpb64, c->lams64, c->lamc64, c->G64};
-    e = launch_step<double>(c->g, tb, c->tiles64, rp, static_cast<const double*>(ucur), static_cast<double*>(uoth),
-                            static_cast<double*>(uoth), nullptr, static_cast<const double*>(c->phi2), c->S,
-                            static_cast<double*>(c->W), st, ev);
+    e = uses_direct64(c)
+            ? dir_step64(c, c->n, static_cast<const double*>(ucur), static_cast<double*>(uoth),
+                         static_cast<double*>(uoth), c->S, static_cast<double*>(c->W), st, ev)
+            : launch_step<double>(c->g, tb, c->tiles64, rp, static_cast<const double*>(ucur),
+                                  static_cast<double*>(uoth), static_cast<double*>(uoth), nullptr,
+                                  static_cast<const double*>(c->phi2), c->S, static_cast<double*>(c->W), st, ev);
   } else {
     StepTables<float> tb{c->stw32, c->tw32, c->lpb32, c->lams32, c->lamc32, c->G32, c3_of(c)};
     float* hi = static_cast<float*>(c->ubuf[0]);
@@ -604,7 +706,15 @@ sadi_status step_reg_group(sadi_ctx* const* cs, int count, cudaStream_t st_) {
   cudaEvent_t* ev = nullptr;
   sadi_status st = next_events(c, &ev);
   if (st != SADI_OK) return st;
-  const cudaError_t e = launch_step_reg(b, c->g.logNp, max_n, st_, ev);
+  // the sweeps of small grids far below their FFT length: dense products
+  const bool direct = dir_mode(c->g, false) == 1;
+  cudaError_t e = launch_step_reg(b, c->g.logNp, blk_path(c->g.logNp, false), max_n, st_, ev, direct);
+  if (direct && e == cudaSuccess) {
+    static thread_local DirBatch<float> d;
+    d.count = count;
+    for (int k = 0; k < count; ++k) d.in[k] = dir_inst32(cs[k]);
+    e = launch_dir_sweeps<float>(d, max_n, st_, ev);
+  }
   if (e != cudaSuccess) {
     for (int k = 0; k < count; ++k) cuda_fail(cs[k], e, "step launch");
     return SADI_ECUDA;
@@ -631,7 +741,7 @@ sadi_status step_dense_group(sadi_ctx* const* cs, int count, cudaStream_t st_) {
       b.in[k] = reg_inst(cs[k]);
       if (cs[k]->g.N > max_n) max_n = cs[k]->g.N;
     }
-    e = launch_step_reg(b, c->g.logNp, max_n, st_, ev, true);
+    e = launch_step_reg(b, c->g.logNp, blk_path(c->g.logNp, true), max_n, st_, ev, true);
   } else {
     // shared-memory engine: the FFT part one member after another (a
     // profiled group has one member, so the events time its kernels), then
@@ -788,6 +898,7 @@ sadi_status batch_issue(sadi_ctx** ctxs, int count, int nsteps) {
     bool placed = false;
     for (auto& gr : groups)
       if (gr[0]->g.logNp == c->g.logNp && is_dense(gr[0]) == is_dense(c) && gr[0]->reg_path == c->reg_path &&
+          (is_dense(c) || dir_mode(gr[0]->g, false) == dir_mode(c->g, false)) &&
           (int)gr.size() < kMaxBatch) {
         gr.push_back(c);
         placed = true;
@@ -1048,7 +1159,7 @@ sadi_status sadi_set_tiles(sadi_ctx* c, int rows, int conv_cols, int solve_cols)
   c->tiles_explicit = was_explicit;
   if (!f64 && !dflt && t.conv_cols == kConvThreePass && (reg || !conv3_supported(c->g.logNp)))
     return fail(c, SADI_EINVAL, "the three-pass convolution serves FFT lengths 2048 .. 8192");
-  if (reg != c->reg_path && is_dense(c) && c->g.logNp == kBlkMinLog && (c->initialized || c->F))
+  if (reg != c->reg_path && is_dense(c) && c->g.logNp == kTilesMinLog && (c->initialized || c->F))
     return fail(c, SADI_ESTATE,
                 "tiles that change the FFT engine (dense form, N' = 2048) must precede sadi_set_initial and "
                 "sadi_set_source");
@@ -1058,8 +1169,14 @@ sadi_status sadi_set_tiles(sadi_ctx* c, int rows, int conv_cols, int solve_cols)
     const sadi_status s3 = ensure_conv3(c);
     if (s3 != SADI_OK) return s3;
   }
-  if (f64) c->tiles64 = t;
-  else c->tiles32 = t;
+  if (f64) {
+    c->tiles64 = t;
+    // tiles equal to the defaults leave the direct path of small grids on
+    const Tiles d = default_tiles<double>(c->g.Np, c->g.N);
+    c->tiles64_explicit = t.rows != d.rows || t.conv_cols != d.conv_cols || t.solve_cols != d.solve_cols;
+  } else {
+    c->tiles32 = t;
+  }
   return SADI_OK;
 }
 
@@ -1207,7 +1324,9 @@ extern "C" sadi_status sadi_step_noalloc(sadi_ctx* c, const double* u_prev, cons
   const size_t nn = (size_t)g.N * g.N;
   const size_t s_bytes = (size_t)g.N * g.Np * 2 * sizeof(double);
   const size_t w_off = (s_bytes + 255) & ~size_t(255);
-  const size_t need = w_off + nn * sizeof(double);
+  const bool direct = uses_direct64(c);   // small grids: V and Wm in place of the spectrum
+  const size_t d_off = ((3 * (size_t)g.N + 2) * g.ld * sizeof(double) + 255) & ~size_t(255);
+  const size_t need = (direct ? d_off : w_off) + nn * sizeof(double);
   if (need > kNoallocScratchBytes)
     return fail(c, SADI_EINVAL,
                 "sadi_step_noalloc: this N needs " + std::to_string(need) + " bytes of scratch, above the fixed " +
@@ -1235,7 +1354,11 @@ extern "C" sadi_status sadi_step_noalloc(sadi_ctx* c, const double* u_prev, cons
   }
   const RhsParams rp = rhs_of(c, n);
   StepTables<double> tb{c->stw64, c->tw64, c->lpb64, c->lams64, c->lamc64, c->G64};
-  double* W = reinterpret_cast<double*>(static_cast<char*>(scratch) + w_off);
+  double* W = reinterpret_cast<double*>(static_cast<char*>(scratch) + (direct ? d_off : w_off));
+  if (direct) {
+    CK(dir_step64(c, n, u_cur, const_cast<double*>(u_prev), u_next, scratch, W, c->stream, nullptr), "step launch");
+    return SADI_OK;
+  }
   // u_prev is only read by the plain (uncompensated) leapfrog form
   CK(launch_step<double>(g, tb, c->tiles64, rp, u_cur, const_cast<double*>(u_prev), u_next, nullptr,
                          static_cast<const double*>(c->phi2), scratch, W, c->stream, nullptr),
@@ -1258,9 +1381,10 @@ extern "C" sadi_status sadi_step_source(sadi_ctx* c, const void* f, int dtype) {
   const bool f64 = c->prec == SADI_PREC_FP64;
   const int N = c->g.N, ld = c->g.ld;
   const void* field = f;
-  // the caller's field is used in place when its type and row pitch are the
-  // context's; else it is converted (and its rows spread to the padded pitch)
-  if ((dtype == 0) != f64 || ld != N) {
+  // the caller's field is used in place when its type is the context's and the
+  // step's kernels take its row pitch (the register paths take any); else it
+  // is converted (and its rows spread to the padded pitch)
+  if ((dtype == 0) != f64 || (ld != N && !c->reg_path)) {
     if (!c->Fconv) CK(cudaMalloc(&c->Fconv, (size_t)ld * N * esize(c->prec)), "cudaMalloc(source conversion)");
     if (f64)
       CK(launch_convert_f2d(static_cast<const float*>(f), static_cast<double*>(c->Fconv), N, N, N, ld, c->stream),

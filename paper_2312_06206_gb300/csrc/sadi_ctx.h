@@ -47,6 +47,9 @@ struct sadi_ctx {
   float2* rlamc = nullptr;
   float2* rlams = nullptr;
   bool reg_path = false;
+  // direct path of small grids (dir_mode), element type per prec: F, T and E
+  void *dF = nullptr, *dT = nullptr, *dE = nullptr;
+  bool tiles64_explicit = false;   // explicit FP64 tiles select the shared-memory engine
   double* lpb64 = nullptr;   // (Np+1) 2 Np
   float* lpb32 = nullptr;
   double2* lamc64 = nullptr;

@@ -36,7 +36,8 @@ struct RhsParams {
   double tau, tau2;
   int g;
   int first;
-  const void* F;   // optional source field (T, N x N) or nullptr
+  const void* F;   // optional source field (T, N x N, row pitch ldF) or nullptr
+  int ldF;         // the state's pitch, or N for a caller's field (register paths)
   double fsc;      // its time factor cos(omega t_n + phase) for this step
   double gc1, gc3, gcs;   // coefficients of g kind 3
 };
@@ -149,16 +150,15 @@ cudaError_t step_setup_attributes();
 // batch:
 // natural-order tables and the in-place double-float state.
 struct RegInst {
-  // [N'] first-level FFT twiddles exp(-2 pi i t k1 / N') at [k1 * T + t], T
-  // threads per vector (T = TT of regfft.cuh, or of blkfft.cuh from N' = 2048 on)
-  const float2* tw1;
-  const float2* tw2;    // second-level twiddles of blkfft.cuh at [k2 * R3 + t'] (N' >= 2048)
-  const float2* tw1h;   // [N'] tw1 at half frequencies: exp(-2 pi i t (k1 + 1/2) / N') (N' >= 2048)
+  const float2* tw1;    // [N'] two-level FFT twiddles exp(-2 pi i t k1 / N') at [k1 * TT + t] (regfft.cuh)
+  // tables of blkfft.cuh: [N'] exp(-2 pi i t k1 / N') at [k1 * T + t], the same
+  // at half frequencies (k1 + 1/2), and the second level's at [k2 * R3 + t']
+  const float2 *btw1, *btw1h, *btw2;
   const float2* tw;     // [2N'] exp(-2 pi i k / 2N')
   const float2* lam_s;  // [N'] natural order, scaled as the bit-reversed tables
   const float2* lam_c;  // [N']
-  const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled (N' <= 1024)
-  const float* lnat;    // [(N'+1) * (N'+1)] symbol by x- and y-frequency 0 .. N', scaled (N' >= 2048)
+  const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled (kRegMaxLog)
+  const float* lnat;    // [(N'+1) * (N'+1)] symbol by x- and y-frequency 0 .. N', scaled (kBlkMinLog)
   const float* G;       // [r * N] border correction, column q at G + q N
   float* u_hi;          // state: u = u_hi + u_lo (double-float), u_d = u^n - u^{n-1}
   float* u_lo;
@@ -168,7 +168,8 @@ struct RegInst {
   int lds;              // rows per slot, N rounded up to 8 (64-byte runs of a cluster's rows stay aligned)
   float* W;             // N x N sweep scratch (by columns between the GS sweeps from N' = 2048 on)
   float* YB;            // bottom entries of the sweeps' bordered solves, r x ld (r > kBorderInline)
-  const float* F;       // optional source field (N x N) or nullptr
+  const float* F;       // optional source field (N x N, row pitch ldF) or nullptr
+  int ldF;
   float* C_hi;          // incremental remainder -kappa tau^2 L_h u^n (double-float)
   float* C_lo;
   unsigned short* Bh;   // dense-inverse form: BF16 split of B^n (ld ldp, zero-padded)
@@ -179,7 +180,7 @@ struct RegInst {
   int* dep;
   int ndep;
   int N, r;
-  int ld;               // row pitch (elements) of the N x N arrays: u_hi, u_lo, u_d, phi2, W, F, C_hi, C_lo
+  int ld;               // row pitch (elements) of the N x N arrays: u_hi, u_lo, u_d, phi2, W, C_hi, C_lo
   float tau, tau2;
   float fsc;            // time factor of the source for this step
   int gkind, first;
@@ -195,6 +196,18 @@ struct RegBatch {
   int count;
   RegInst in[kMaxBatch];
 };
+// FFT lengths of the two register paths: step_reg.cuh (a row per part of a warp)
+// up to 2^kRegMaxLog, step_blk.cuh (a row per warp or more) from 2^kBlkMinLog;
+// explicit tiles select the shared-memory engine from 2^kTilesMinLog on.
+constexpr int kRegMaxLog = 10, kBlkMinLog = 8, kTilesMinLog = 11;
+// whether step_blk.cuh serves a context, else step_reg.cuh.  From N' = 256 on it
+// measured faster for one instance and for many (us per step, step_reg.cuh ->
+// step_blk.cuh: GS N = 255 1 / 16 instances 31 -> 21 / 63 -> 58, N = 511 68 ->
+// 29 / 240 -> 201, N = 1023 91 -> 62 / 981 -> 774; dense N = 511 72 -> 45), but
+// for the dense form's row kernels at N' = 1024, whose 21-row blocks have one
+// exchange per transform (three instances: row FFT 12.3 against 18, B^n 30
+// against 45; the column convolution is step_blk.cuh's there too).
+inline bool blk_path(int logNp, bool dense) { return logNp >= kBlkMinLog && !(dense && logNp == 10); }
 // whether a context of FFT length 2^logNp and precision prec (SADI_PREC_*)
 // can step on the register path
 bool reg_path_supported(int logNp, int prec);
@@ -202,19 +215,63 @@ bool reg_path_supported(int logNp, int prec);
 // max_n = the largest N in the batch.  dense: only the row FFT, the column
 // convolution and the B^n kernel run (events 0..2), the latter writing B^n to
 // W and its BF16 split to Bh / Bl; the sweeps are left to the GEMMs.
-cudaError_t launch_step_reg(const RegBatch& b, int logNp, int max_n, cudaStream_t st, cudaEvent_t* ev,
+cudaError_t launch_step_reg(const RegBatch& b, int logNp, bool blk, int max_n, cudaStream_t st, cudaEvent_t* ev,
                             bool dense = false);
 // natural-order FP32 tables of the register paths from the FP64 setup
-// products: tw1 (N' entries) followed by tw2 (kTw2) and tw1h (N'), and the symbol
-// (reg_symbol_elems floats: RegInst::lreg or ::lnat by FFT length)
+// products, behind one another in tw: tw1 (N' entries, step_reg.cuh), btw1
+// (N'), btw1h (N'), btw2 (kTw2); and in sym: lreg (reg_lreg_elems floats) and
+// lnat (reg_lnat_elems), each where its path exists
 constexpr int kTw2 = 256;
-constexpr int kBlkMinLog = 11;   // first log2 N' of the block-wide FFT
-inline size_t reg_symbol_elems(const Geom& g) {
-  return g.logNp >= kBlkMinLog ? (size_t)(g.Np + 1) * (g.Np + 1) : (size_t)(g.Np + 1) * 2 * g.Np;
-}
+inline size_t reg_lreg_elems(const Geom& g) { return g.logNp <= kRegMaxLog ? (size_t)(g.Np + 1) * 2 * g.Np : 0; }
+inline size_t reg_lnat_elems(const Geom& g) { return g.logNp >= kBlkMinLog ? (size_t)(g.Np + 1) * (g.Np + 1) : 0; }
 cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, const double2* lamc64,
-                           const double2* lams64, float2* tw1, float* lreg, float2* lamc_nat, float2* lams_nat,
+                           const double2* lams64, float2* tw, float* sym, float2* lamc_nat, float2* lams_nat,
                            cudaStream_t st);
+
+// ---- direct path of small grids, step_dir.cu -------------------------------------
+// One instance: tables (run_dir_tables; E, N x N), the field whose convolution
+// the step takes (FP64: u + beta (u - x2)), scratch and state.  FP32: u = next
+// = u_hi, aux = d, lo = u_lo; FP64: u = u^n, aux = u^{n-1}, next = u^{n+1} (may
+// be aux).
+template <typename T>
+struct DirInst {
+  const T *F, *T_, *E;
+  const T *x, *x2;
+  T beta;
+  T* V;      // (2N + 2) x ld
+  T* Bm;     // N x ld: B^n
+  T* Wm;     // N x ld: x-sweep result
+  const T* u;
+  T *aux, *next, *lo;
+  const T *phi2, *src;
+  int ident;   // E holds H^-1 - I, else H^-1
+  int N, ld, gkind, first, eq;
+  T tau, tau2, fsc, gc1, gc3, gcs;
+};
+template <typename T>
+struct DirBatch {
+  int count;
+  DirInst<T> in[kMaxBatch];
+};
+// what the direct path computes for an FP64 or FP32 (GS) context: 0 nothing, 1
+// the two sweeps, 2 the whole step
+inline int dir_mode(const Geom& g, bool fp64) {
+  if (fp64) return g.logNp <= 7 ? 2 : 0;
+  return g.r > kBorderInline && g.logNp <= 9 ? 1 : 0;
+}
+// F ((2N + 2) x N) and T ((N + 1) x N, scale = -kappa tau^2 h^-alpha)
+cudaError_t run_dir_tables(double* F, double* Tk, const double* a2d, int N, double scale, cudaStream_t st);
+// E = H^-1 - I (ident) or H^-1, N rows of pitch ld (the padding zeroed by the
+// caller), from the generator of the N x N matrix; *status_host as
+// run_generator
+template <typename T>
+cudaError_t run_dir_inverse(const double* a1, int N, int ld, double s, bool ident, T* E, int* status_host,
+                            cudaStream_t st);
+// one step of every instance / its two sweeps alone (B^n in Bm); events as
+// launch_step (the sweeps record 3 and 4)
+cudaError_t launch_dir_step(const DirBatch<double>& b, int max_n, cudaStream_t st, cudaEvent_t* ev);
+template <typename T>
+cudaError_t launch_dir_sweeps(const DirBatch<T>& b, int max_n, cudaStream_t st, cudaEvent_t* ev);
 
 // One S-ADI step: u_next (may alias u_prev) from u_cur, u_prev.
 // S: N x Np complex scratch, W: N x N scratch.
@@ -356,10 +413,13 @@ cudaError_t noalloc_scratch_address(int device, void** out);
 // ---- programmatic dependent launch of the shared-memory engine's kernels ------
 // launch_dependent starts `kernel` on st as a programmatic dependent of the
 // kernel before it in the stream: its blocks may be scheduled before that
-// kernel has finished.  Every kernel launched this way opens with
-// pdl_entry(), which lets the kernel after it be scheduled likewise and then
-// waits until the kernel before it has completed and its writes are visible
-// (a no-op for a launch without the attribute).  Every argument is passed
+// kernel has finished.  Every kernel launched this way calls pdl_entry() before
+// it touches anything an earlier kernel writes: it waits until the kernel
+// before it has completed and its writes are visible, then lets the kernel
+// after it be scheduled (a no-op for a launch without the attribute).  In this
+// order one kernel at most waits beside a running one; letting the dependent
+// in first piled up whole steps of waiting blocks on small grids (N = 255 FP32
+// step 20.8 -> 17.6 us, N = 63 FP64 21.6 -> 16.0).  Every argument is passed
 // explicitly (default arguments do not apply through the pointer).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
@@ -379,8 +439,8 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_entry() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
 

@@ -358,44 +358,34 @@ __global__ void k_border_G(const double* __restrict__ X, const double* __restric
   G32[at] = (float)(-acc);
 }
 
-// Register-path tables.  tw1: exp(-2 pi i t k1 / Np) at [k1 * T + t] (T: threads
-// per vector), from N' = 2048 on followed by tw2, exp(-2 pi i t' k2 / T) at
-// [k2 * R3 + t'], and tw1h, exp(-2 pi i t (k1 + 1/2) / Np) at [k1 * T + t].  Symbol, scaled: up to N' = 1024 lreg[(k1 * 2 + h) * Np + m] =
-// Lambda(k1, 2m + h) (k2 folded into [0, Np]), above lnat32[k1 * (Np + 1) + k2].
+// Register-path tables (layout: run_reg_tables).  TT, T: threads per vector of
+// regfft.cuh and blkfft.cuh (T = 0: no block path at this length).
 // lam*_nat[k] = lam*[brev(k)].
-__global__ void k_reg_tables(Geom g, const double* __restrict__ lnat, double scale, int T, int R3,
-                             const double2* __restrict__ lamc64, const double2* __restrict__ lams64, float2* tw1,
-                             float* lreg, float2* lamc_nat, float2* lams_nat) {
+__global__ void k_reg_tables(Geom g, const double* __restrict__ lnat, double scale, int TT, int T, int R3,
+                             const double2* __restrict__ lamc64, const double2* __restrict__ lams64, float2* tw,
+                             float* lreg, size_t nreg, float* lfold, size_t nfold, float2* lamc_nat, float2* lams_nat) {
   const int Np = g.Np, logNp = g.logNp, P = g.P;
-  const bool folded = R3 > 0;
-  const size_t nl = folded ? (size_t)(Np + 1) * (Np + 1) : (size_t)(Np + 1) * 2 * Np;
   const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  auto root = [](double num, double den) {   // exp(-2 pi i num / den)
+    double s, c;
+    sincospi(2.0 * num / den, &s, &c);
+    return make_float2((float)c, (float)-s);
+  };
   if (idx < (size_t)Np) {
     const int k = (int)idx;
-    const int t = k % T, k1 = k / T;
-    double sn, cs;
-    sincospi(2.0 * (double)((long long)t * k1 % Np) / (double)Np, &sn, &cs);
-    tw1[k] = make_float2((float)cs, (float)-sn);
-    if (folded) {
-      sincospi((double)((long long)t * (2 * k1 + 1) % P) / (double)Np, &sn, &cs);
-      tw1[Np + kTw2 + k] = make_float2((float)cs, (float)-sn);
+    tw[k] = root((double)((long long)(k % TT) * (k / TT) % Np), (double)Np);
+    if (T) {
+      const long long t = k % T, k1 = k / T;
+      tw[Np + k] = root((double)(t * k1 % Np), (double)Np);
+      tw[2 * Np + k] = root((double)(t * (2 * k1 + 1) % P), (double)P);
+      if (k < T) tw[3 * Np + k] = root((double)((k % R3) * (k / R3)), (double)T);
     }
     const double2 a = lamc64[brev(k, logNp)], b = lams64[brev(k, logNp)];
     lamc_nat[k] = make_float2((float)a.x, (float)a.y);
     lams_nat[k] = make_float2((float)b.x, (float)b.y);
   }
-  if (folded && idx < (size_t)T) {
-    const int k = (int)idx;
-    const int t = k % R3, k2 = k / R3;
-    double sn, cs;
-    sincospi(2.0 * (double)(t * k2) / (double)T, &sn, &cs);
-    tw1[Np + k] = make_float2((float)cs, (float)-sn);
-  }
-  if (idx < nl) {
-    if (folded) {
-      lreg[idx] = (float)(scale * lnat[idx]);
-      return;
-    }
+  if (idx < nfold) lfold[idx] = (float)(scale * lnat[idx]);
+  if (idx < nreg) {
     const int m = (int)(idx % Np);
     const int h = (int)((idx / Np) % 2);
     const int k1 = (int)(idx / (2 * (size_t)Np));
@@ -461,10 +451,10 @@ cudaError_t launch_stage_twiddles(double2* stw64, float2* stw32, int logL, cudaS
 }
 
 cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, const double2* lamc64,
-                           const double2* lams64, float2* tw1, float* lreg, float2* lamc_nat, float2* lams_nat,
+                           const double2* lams64, float2* tw, float* sym, float2* lamc_nat, float2* lams_nat,
                            cudaStream_t st) {
-  const size_t nl = reg_symbol_elems(g);
-  int T = 1 << (g.logNp / 2), R3 = 0;
+  const size_t nreg = reg_lreg_elems(g), nfold = reg_lnat_elems(g);
+  int T = 0, R3 = 1;
   auto blk = [&](auto f) {
     using F = decltype(f);
     static_assert(F::T <= kTw2, "room for tw2");
@@ -472,12 +462,17 @@ cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, cons
     R3 = F::R3;
   };
   switch (g.logNp) {
+    case 8: blk(bf::BlkFFT<8>{}); break;
+    case 9: blk(bf::BlkFFT<9>{}); break;
+    case 10: blk(bf::BlkFFT<10>{}); break;
     case 11: blk(bf::BlkFFT<11>{}); break;
     case 12: blk(bf::BlkFFT<12>{}); break;
     case 13: blk(bf::BlkFFT<13>{}); break;
     default: break;
   }
-  k_reg_tables<<<nblk(nl, 256), 256, 0, st>>>(g, lnat, scale, T, R3, lamc64, lams64, tw1, lreg, lamc_nat, lams_nat);
+  const size_t n = nreg > nfold ? nreg : nfold;
+  k_reg_tables<<<nblk(n, 256), 256, 0, st>>>(g, lnat, scale, 1 << (g.logNp / 2), T, R3, lamc64, lams64, tw, sym, nreg,
+                                             sym + nreg, nfold, lamc_nat, lams_nat);
   return cudaGetLastError();
 }
 
@@ -521,9 +516,9 @@ cudaError_t launch_convert_f2d(const float* s, double* d, int rows, int cols, in
 // y = (0, c_{n-1}, ..., c_1), read along diagonals:
 //   (H^-1)[d + j][j] = (H^-1)[d + j - 1][j - 1] + (c_{d+j} c_j - y_{d+j} y_j) / c_0,
 //   (H^-1)[d][0] = c_d.
-// One thread per diagonal d; both triangles written (symmetry), as BF16 pairs.
-__global__ void k_dense_inverse(const double* __restrict__ c, int n, int npad, unsigned short* Eh,
-                                unsigned short* El) {
+// One thread per diagonal d; both triangles written (symmetry) through put(i, j, e).
+template <typename Put>
+__device__ __forceinline__ void inverse_diagonal(const double* __restrict__ c, int n, Put put) {
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= n) return;
   const double c0 = c[0];
@@ -531,16 +526,22 @@ __global__ void k_dense_inverse(const double* __restrict__ c, int n, int npad, u
   for (int j = 0; j < n - d; ++j) {
     if (j > 0) v += (c[d + j] * c[j] - c[n - d - j] * c[n - j]) / c0;
     const double e = (d == 0) ? v - 1.0 : v;
-    const float ef = (float)e;
-    const __nv_bfloat16 h = __float2bfloat16_rn(ef);
-    const unsigned short hb = __bfloat16_as_ushort(h);
-    const unsigned short lb = __bfloat16_as_ushort(__float2bfloat16_rn((float)(e - (double)__bfloat162float(h))));
-    const size_t a = (size_t)(d + j) * npad + j, b = (size_t)j * npad + (d + j);
-    Eh[a] = hb;
-    El[a] = lb;
-    Eh[b] = hb;
-    El[b] = lb;
+    put(d + j, j, e);
+    put(j, d + j, e);
   }
+}
+__global__ void k_dense_inverse(const double* __restrict__ c, int n, int npad, unsigned short* Eh,
+                                unsigned short* El) {
+  inverse_diagonal(c, n, [&](int i, int j, double e) {
+    const __nv_bfloat16 h = __float2bfloat16_rn((float)e);
+    const size_t a = (size_t)i * npad + j;
+    Eh[a] = __bfloat16_as_ushort(h);
+    El[a] = __bfloat16_as_ushort(__float2bfloat16_rn((float)(e - (double)__bfloat162float(h))));
+  });
+}
+template <typename T>
+__global__ void k_dir_inverse(const double* __restrict__ c, int n, int ld, int ident, T* E) {
+  inverse_diagonal(c, n, [&](int i, int j, double e) { E[(size_t)i * ld + j] = (T)(i == j && !ident ? e + 1.0 : e); });
 }
 
 #define SADI_TRY(x)                        \
@@ -680,5 +681,28 @@ done:
   cudaFree(c);
   return err;
 }
+
+template <typename T>
+cudaError_t run_dir_inverse(const double* a1, int N, int ld, double s, bool ident, T* E, int* status_host, cudaStream_t st) {
+  cudaError_t err = cudaSuccess;
+  int* dstat = nullptr;
+  double* c = nullptr;
+  *status_host = 1;
+  SADI_TRY(cudaFuncSetAttribute(k_durbin, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  SADI_TRY(cudaMalloc(&dstat, sizeof(int)));
+  SADI_TRY(cudaMalloc(&c, sizeof(double) * N));
+  k_durbin<<<1, 1024, sizeof(double) * (2 * (size_t)N + 1 + 32), st>>>(a1, N, s, c, dstat);
+  SADI_TRY(cudaGetLastError());
+  k_dir_inverse<T><<<nblk(N, 32), 32, 0, st>>>(c, N, ld, ident ? 1 : 0, E);
+  SADI_TRY(cudaGetLastError());
+  SADI_TRY(cudaMemcpyAsync(status_host, dstat, sizeof(int), cudaMemcpyDeviceToHost, st));
+  SADI_TRY(cudaStreamSynchronize(st));
+done:
+  cudaFree(dstat);
+  cudaFree(c);
+  return err;
+}
+template cudaError_t run_dir_inverse<float>(const double*, int, int, double, bool, float*, int*, cudaStream_t);
+template cudaError_t run_dir_inverse<double>(const double*, int, int, double, bool, double*, int*, cudaStream_t);
 
 }  // namespace sadi

@@ -87,12 +87,6 @@ __device__ __forceinline__ void cluster_join() {
   cluster_arrive_relaxed();
   cluster_wait();
 }
-// address of p (this block's shared memory) in block `rank` of the cluster
-__device__ __forceinline__ unsigned peer(const void* p, int rank) {
-  unsigned r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
-  return r;
-}
 __device__ __forceinline__ void st_peer(unsigned a, float2 v) {
   asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
@@ -100,50 +94,96 @@ __device__ __forceinline__ void st_peer(unsigned a, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 
+// Barrier of the T threads of a row (rl: the row's place in its block).
+template <int T>
+__device__ __forceinline__ void row_sync(int rl) {
+  if constexpr (T == 32) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(1 + rl), "n"(T) : "memory");
+}
+
 template <int LOGL>
 struct Cfg {
   using F = BlkFFT<LOGL>;
   static constexpr int V = kCluster;
+  // rows per block: short rows share one, which needs fewer or no distributed
+  // exchanges (us per step, 1 / 16 instances at 1, 2, 4, 8 rows a block: GS N =
+  // 511 32 / 238, 32 / 231, 31 / 219, 29 / 201; N = 1023 64 / 840, 62 / 817, 62 /
+  // 774 (4); at N = 2047 four rows measured slower than one, 246 against 224)
+  static constexpr int R = LOGL <= 9 ? 8 : LOGL == 10 ? 4 : 1;
+  static constexpr int CL = V / R;                   // blocks per cluster
   static constexpr int SEG = F::L / V;               // frequencies (columns) per block of the exchange
   static constexpr int QS = F::E / V;                // registers q per segment: t + T q lies in segment q / QS
   static_assert(SEG % F::T == 0 && QS * V == F::E, "whole register groups per segment");
   // row pitches of the exchange buffers: a half-warp (8-byte) or a warp
   // (4-byte) reading V rows x 16/V (32/V) neighbours finds distinct banks
   static constexpr int P2 = SEG + 16 / V, P1 = SEG + 32 / V;
-  static_assert(V * P2 <= F::BUF && V * P1 <= 2 * F::BUF, "exchange buffers inside the transform buffer");
-  static constexpr size_t bytes = (size_t)F::BUF * sizeof(float2);
-  static constexpr size_t bytes_conv = 2 * bytes;
+  // transform buffer and exchange buffers share the space
+  static constexpr int ELEMS = F::BUF > V * P2 ? F::BUF : V * P2;
+  static_assert(V * P1 <= 2 * ELEMS, "the float exchange buffer fits too");
+  static constexpr size_t bytes = (size_t)R * ELEMS * sizeof(float2);
+  static constexpr size_t bytes_conv = 2 * (size_t)F::BUF * sizeof(float2);
   // resident blocks promised to the compiler (its register budget), measured
   // at N = 4095 (us per launch at 2 / 3 / 4 blocks of 256 threads): r2c 109 /
   // 100 / 94, dense B^n 208 / 179 / 177, GS rows 378 / 362 / -, columns
   // 289 / 312, convolution 193 (one block of 512 threads, 128 registers)
   // against 219 (two, 64 registers).  E = 32 (N' = 8192) needs 128 registers.
-  static constexpr int kM = LOGL == 11 ? 2 : 1;   // half the threads per block
-  static constexpr int kR2cBlocks = LOGL == 13 ? 2 : 4 * kM;
-  static constexpr int kDenseBlocks = LOGL == 13 ? 2 : 4 * kM;
-  static constexpr int kGsBlocks = LOGL == 13 ? 2 : 3 * kM;
-  static constexpr int kColsBlocks = 2 * kM;
-  static constexpr int kConvBlocks = kM;
+  static constexpr int kM = 256 / F::T;   // rows for each 256 threads
+  static constexpr int per(int rows) { return rows / R > 0 ? rows / R : 1; }
+  static constexpr int kR2cBlocks = per(LOGL == 13 ? 2 : 4 * kM);
+  static constexpr int kDenseBlocks = per(LOGL == 13 ? 2 : LOGL >= 11 ? 4 * kM : 2 * kM);
+  static constexpr int kGsBlocks = per(LOGL == 13 ? 2 : LOGL >= 11 ? 3 * kM : 2 * kM);
+  static constexpr int kColsBlocks = per(2 * kM);
+  static constexpr int kConvBlocks = LOGL >= 11 ? kM : F::E == 8 ? 2 * kM : kM;
 };
 
-__device__ __forceinline__ void pdl_allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Exchange between the V rows of a cluster: barriers over all of them and the
+// address of p (in the calling row's buffer) in the buffer of row `to`.
+template <int LOGL>
+struct Exchange {
+  using C = Cfg<LOGL>;
+  __device__ static __forceinline__ void join() {   // no release: see cluster_join
+    if constexpr (C::CL == 1) __syncthreads();
+    else cluster_join();
+  }
+  __device__ static __forceinline__ void sync() {
+    if constexpr (C::CL == 1) __syncthreads();
+    else cluster_sync();
+  }
+  template <typename P>
+  __device__ static __forceinline__ unsigned at(const P* p, int rl, int to) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p) + (unsigned)((to % C::R - rl) * (int)(C::ELEMS * sizeof(float2)));
+    if constexpr (C::CL == 1) return a;
+    unsigned r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(to / C::R));
+    return r;
+  }
+  template <typename T>
+  __device__ static __forceinline__ void put(unsigned a, T v) {
+    if constexpr (C::CL > 1) st_peer(a, v);
+    else if constexpr (sizeof(T) == 8) asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+    else asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+  }
+};
+
+__device__ __forceinline__ void pdl_wait_prerequisites() { pdl_entry(); }
 
 // ---------------------------------------------------------------------------
 template <int LOGL>
-__global__ void __launch_bounds__(BlkFFT<LOGL>::T, Cfg<LOGL>::kR2cBlocks)
+__global__ void __launch_bounds__(Cfg<LOGL>::R * BlkFFT<LOGL>::T, Cfg<LOGL>::kR2cBlocks)
 kb_rows_r2c(const __grid_constant__ RegBatch B) {
   using F = BlkFFT<LOGL>;
   using C = Cfg<LOGL>;
+  using X = Exchange<LOGL>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* sm = reinterpret_cast<float2*>(smem_raw);
-  pdl_allow_dependents();
+  // row rl of the block, thread t of the row
+  const int rl = C::R == 1 ? 0 : threadIdx.x / F::T, t = C::R == 1 ? threadIdx.x : threadIdx.x % F::T;
+  float2* sm = reinterpret_cast<float2*>(smem_raw) + rl * C::ELEMS;
   const RegInst& I = B.in[blockIdx.y];
-  const int N = I.N, t = threadIdx.x;
-  const int rank = blockIdx.x % C::V, row0 = blockIdx.x - rank, row = blockIdx.x;
+  const int N = I.N;
+  const int row = blockIdx.x * C::R + rl, rank = row % C::V, row0 = row - rank;
   if (row0 >= N) return;   // the whole cluster
   const bool valid = row < N;
-  auto sync = [] { __syncthreads(); };
+  auto sync = [rl] { C::R == 1 ? __syncthreads() : row_sync<F::T>(rl); };
   pdl_wait_prerequisites();
   // z[n] = d[2n] + i d[2n+1], zero from n = N'/2 on (2n < N <= N'); an even
   // offset in a 128-byte aligned row: 8-byte loads, row padding beyond N - 1
@@ -159,7 +199,7 @@ kb_rows_r2c(const __grid_constant__ RegBatch B) {
     }
     x[q] = v;
   });
-  F::fwd(x, sm, t, I.tw1, false, I.tw2, sync);
+  F::fwd(x, sm, t, I.btw1, false, I.btw2, sync);
   static_for<0, F::E>([&](auto qc) { sm[t + F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
   sync();
   // X[k] = (Z[k] + conj Z[-k]) / 2 + w^k (Z[k] - conj Z[-k]) / (2 i); slot 0 = X[0] + i X[N']
@@ -171,16 +211,16 @@ kb_rows_r2c(const __grid_constant__ RegBatch B) {
     const float2 Ov = cscale(cmul_mi(csub(Z, Zc)), 0.5f);
     x[q] = (q == 0 && t == 0) ? make_float2(Ev.x + Ov.x, Ev.x - Ov.x) : cadd(Ev, cmul(__ldg(&I.tw[k]), Ov));
   });
-  cluster_join();   // every block of the cluster has read its buffer
+  X::join();   // every row of the cluster has read its buffer
   static_for<0, C::V>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
-    const unsigned dst = peer(sm + rank * C::P2 + t, c);
+    const unsigned dst = X::at(sm + rank * C::P2 + t, rl, c);
     static_for<0, C::QS>([&](auto jc) {
       constexpr int j = decltype(jc)::value;
-      st_peer(dst + (unsigned)(F::T * j * sizeof(float2)), x[c * C::QS + j]);
+      X::put(dst + (unsigned)(F::T * j * sizeof(float2)), x[c * C::QS + j]);
     });
   });
-  cluster_sync();   // the rows' segments have arrived
+  X::sync();   // the rows' segments have arrived
   const int vv = t % C::V, s0 = t / C::V;
   if (row0 + vv >= N) return;
   float2* col = I.S + (size_t)(rank * C::SEG + s0) * I.lds + row0 + vv;
@@ -199,7 +239,6 @@ __global__ void __launch_bounds__(2 * BlkFFT<LOGL>::T, Cfg<LOGL>::kConvBlocks)
 kb_cols_conv(const __grid_constant__ RegBatch B) {
   using F = BlkFFT<LOGL>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_allow_dependents();
   const RegInst& I = B.in[blockIdx.y];
   const int N = I.N, kx = blockIdx.x;
   const int h = threadIdx.x / F::T, t = threadIdx.x % F::T;
@@ -224,8 +263,8 @@ kb_cols_conv(const __grid_constant__ RegBatch B) {
     });
   }
   // odd half: frequencies m + 1/2 of the length-L transform
-  const float2* tw1 = h ? I.tw1h : I.tw1;
-  F::fwd(x, sm, t, tw1, h, I.tw2, sync);
+  const float2* tw1 = h ? I.btw1h : I.btw1;
+  F::fwd(x, sm, t, tw1, h, I.btw2, sync);
   // the symbol at y frequency 2 m + h, stored for 0 .. N' (it is even)
   const float* lam = I.lnat + (size_t)kx * (F::L + 1);
   static_for<0, F::E>([&](auto qc) {
@@ -233,7 +272,7 @@ kb_cols_conv(const __grid_constant__ RegBatch B) {
     const int k2 = 2 * (t + F::T * q) + h;
     x[q] = cscale(x[q], __ldg(&lam[q < F::E / 2 ? k2 : 2 * F::L - k2]));
   });
-  F::inv(x, sm, t, tw1, h, I.tw2, sync);
+  F::inv(x, sm, t, tw1, h, I.btw2, sync);
   // even + odd half: the odd threads hand over the rows of
   // q < E/2, the even threads the others, and each finishes its own rows
   constexpr int HE = F::E / 2;
@@ -269,13 +308,13 @@ __device__ __forceinline__ void gs_solve(float2* x, float* y, float2* sm, int t,
 #pragma unroll 1
   for (int round = 0; round < 2; ++round) {
     const float2* lam = round == 0 ? I.lam_s : I.lam_c;
-    const float2* tw1 = round == 0 ? I.tw1h : I.tw1;
-    F::fwd(x, sm, t, tw1, round == 0, I.tw2, sync);
+    const float2* tw1 = round == 0 ? I.btw1h : I.btw1;
+    F::fwd(x, sm, t, tw1, round == 0, I.btw2, sync);
     static_for<0, F::E>([&](auto qc) {
       constexpr int q = decltype(qc)::value;
       x[q] = cmul(x[q], __ldg(&lam[t + F::T * q]));
     });
-    F::inv(x, sm, t, tw1, round == 0, I.tw2, sync);
+    F::inv(x, sm, t, tw1, round == 0, I.btw2, sync);
   }
   static_for<0, F::E>([&](auto qc) { sm[t + F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
   sync();
@@ -306,21 +345,23 @@ __device__ __forceinline__ void gs_solve(float2* x, float* y, float2* sm, int t,
 // and, split into BF16 pairs, to Bh / Bl (the first sweep GEMM's A operand).
 // Else W receives the x sweep by columns, W[k * ld + row].
 template <int LOGL, bool DENSE>
-__global__ void __launch_bounds__(BlkFFT<LOGL>::T, DENSE ? Cfg<LOGL>::kDenseBlocks : Cfg<LOGL>::kGsBlocks)
+__global__ void __launch_bounds__(Cfg<LOGL>::R * BlkFFT<LOGL>::T, DENSE ? Cfg<LOGL>::kDenseBlocks : Cfg<LOGL>::kGsBlocks)
 kb_rows_solve(const __grid_constant__ RegBatch B) {
   using F = BlkFFT<LOGL>;
   using C = Cfg<LOGL>;
+  using X = Exchange<LOGL>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* sm = reinterpret_cast<float2*>(smem_raw);
-  pdl_allow_dependents();
+  // row rl of the block, thread t of the row
+  const int rl = C::R == 1 ? 0 : threadIdx.x / F::T, t = C::R == 1 ? threadIdx.x : threadIdx.x % F::T;
+  float2* sm = reinterpret_cast<float2*>(smem_raw) + rl * C::ELEMS;
   const RegInst& I = B.in[blockIdx.y];
-  const int N = I.N, t = threadIdx.x;
-  const int rank = blockIdx.x % C::V, row0 = blockIdx.x - rank, row = blockIdx.x;
+  const int N = I.N;
+  const int row = blockIdx.x * C::R + rl, rank = row % C::V, row0 = row - rank;
   if (row0 >= N) return;   // the whole cluster
   const bool valid = row < N;
   const size_t rbase = (size_t)(valid ? row : 0) * I.ld;
-  auto sync = [] { __syncthreads(); };
-  cluster_arrive_relaxed();   // peers may be written once every block runs
+  auto sync = [rl] { C::R == 1 ? __syncthreads() : row_sync<F::T>(rl); };
+  if constexpr (C::CL > 1) cluster_arrive_relaxed();   // peers may be written once every block runs
   // the rows the B^n epilogue reads into L2 under the convolution's tail
   // (written in the previous step; a prefetch cannot make a load see older data)
   if (valid) {
@@ -333,7 +374,7 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
   pdl_wait_prerequisites();
   if constexpr (DENSE) {
     // zero the sweep GEMM's counters for the GEMM that follows
-    if (blockIdx.x == 0 && I.dep)
+    if (row == 0 && I.dep)
       for (int i = t; i < I.ndep; i += F::T) I.dep[i] = 0;
   }
   float2 x[F::E];
@@ -346,25 +387,25 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
       constexpr int i = decltype(ic)::value;
       x[i] = ok ? ld_stream(col + (size_t)(F::T / C::V * i) * I.lds) : make_float2(0.f, 0.f);
     });
-    cluster_wait();
-    const unsigned dst = peer(sm + rank * C::SEG + s0, vv);
+    if constexpr (C::CL > 1) cluster_wait();
+    const unsigned dst = X::at(sm + rank * C::SEG + s0, rl, vv);
     static_for<0, F::E>([&](auto ic) {
       constexpr int i = decltype(ic)::value;
-      st_peer(dst + (unsigned)(F::T / C::V * i * sizeof(float2)), x[i]);
+      X::put(dst + (unsigned)(F::T / C::V * i * sizeof(float2)), x[i]);
     });
   }
-  cluster_sync();
+  X::sync();
   // half spectrum X[k] -> Z[k] = E + i O, the spectrum of z[n] = x[2n] + i x[2n+1]
   static_for<0, F::E>([&](auto qc) {
     constexpr int q = decltype(qc)::value;
     const int k = t + F::T * q;
-    const float2 X = sm[k], Xc = cconj(sm[(F::L - k) & (F::L - 1)]);
-    const float2 Ev = cscale(cadd(X, Xc), 0.5f);
-    const float2 Ov = cscale(cmulc(csub(X, Xc), __ldg(&I.tw[k])), 0.5f);
-    x[q] = (q == 0 && t == 0) ? make_float2(0.5f * (X.x + X.y), 0.5f * (X.x - X.y)) : cadd(Ev, cmul_pi(Ov));
+    const float2 Xk = sm[k], Xc = cconj(sm[(F::L - k) & (F::L - 1)]);
+    const float2 Ev = cscale(cadd(Xk, Xc), 0.5f);
+    const float2 Ov = cscale(cmulc(csub(Xk, Xc), __ldg(&I.tw[k])), 0.5f);
+    x[q] = (q == 0 && t == 0) ? make_float2(0.5f * (Xk.x + Xk.y), 0.5f * (Xk.x - Xk.y)) : cadd(Ev, cmul_pi(Ov));
   });
   sync();
-  F::inv(x, sm, t, I.tw1, false, I.tw2, sync);
+  F::inv(x, sm, t, I.btw1, false, I.btw2, sync);
   // x[q], q < E/2, now holds the convolution at 2n, 2n + 1, n = t + T q.
   // Wave step: B = C + tau^2 (g(u) + f), n = 0: tau phi2 + (C + tau^2 (g + f))/2,
   // with C <- C + conv; diffusion: B = C + conv/2 + tau (g(u~) + f) - d,
@@ -372,7 +413,7 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
   const float tau = I.tau, tau2 = I.tau2;
   auto bn = [&](auto diff_c) {
     constexpr bool DIFF = decltype(diff_c)::value;
-    constexpr int HE = F::E / 2, GR = HE < 8 ? HE : 8;
+    constexpr int HE = F::E / 2, GR = HE < 8 ? HE : 8;   // loads in flight per array
     static_for<0, HE / GR>([&](auto gc) {
       constexpr int q0 = decltype(gc)::value * GR;
       float2 ch[GR], cl[GR], uv[GR];
@@ -409,13 +450,13 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
             const float u = e ? uv[j].y : uv[j].x;
             if constexpr (!DIFF) {
               float gs = g_of_b(I, u);
-              if (I.F) gs += I.fsc * I.F[rbase + i];
+              if (I.F) gs += I.fsc * I.F[(size_t)row * I.ldF + i];
               const float gg = tau2 * gs;
               b[e] = I.first ? tau * I.phi2[rbase + i] + 0.5f * (c + gg) : c + gg;
             } else {
               const float d = e ? dv[j].y : dv[j].x;
               float gs = g_of_b(I, u + 0.5f * d);
-              if (I.F) gs += I.fsc * I.F[rbase + i];
+              if (I.F) gs += I.fsc * I.F[(size_t)row * I.ldF + i];
               b[e] = (c + 0.5f * cx) + tau2 * gs - d;
             }
           }
@@ -435,10 +476,12 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
             float* wr = I.W + rbase;
             if (e0 + 1 < N) *reinterpret_cast<float2*>(wr + e0) = make_float2(b[0], b[1]);
             else wr[e0] = b[0];
-            unsigned hi, lo;
-            split_bf16x2(b[0], b[1], &hi, &lo);
-            *reinterpret_cast<unsigned*>(I.Bh + (size_t)row * I.ldp + e0) = hi;
-            *reinterpret_cast<unsigned*>(I.Bl + (size_t)row * I.ldp + e0) = lo;
+            if (I.Bh) {
+              unsigned hi, lo;
+              split_bf16x2(b[0], b[1], &hi, &lo);
+              *reinterpret_cast<unsigned*>(I.Bh + (size_t)row * I.ldp + e0) = hi;
+              *reinterpret_cast<unsigned*>(I.Bl + (size_t)row * I.ldp + e0) = lo;
+            }
           }
         } else {
           sm[t + F::T * (q0 + j)] = make_float2(b[0], b[1]);
@@ -462,17 +505,17 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
     sync();
     float y[F::E];
     gs_solve<LOGL>(x, y, sm, t, row, I, sync);
-    cluster_join();   // every block of the cluster has read its buffer
+    X::join();   // every row of the cluster has read its buffer
     float* smf = reinterpret_cast<float*>(sm);
     static_for<0, C::V>([&](auto cc) {
       constexpr int c = decltype(cc)::value;
-      const unsigned dst = peer(smf + rank * C::P1 + t, c);
+      const unsigned dst = X::at(smf + rank * C::P1 + t, rl, c);
       static_for<0, C::QS>([&](auto jc) {
         constexpr int j = decltype(jc)::value;
-        st_peer(dst + (unsigned)(F::T * j * sizeof(float)), y[c * C::QS + j]);
+        X::put(dst + (unsigned)(F::T * j * sizeof(float)), y[c * C::QS + j]);
       });
     });
-    cluster_sync();
+    X::sync();
     const int vv = t % C::V, s0 = t / C::V;
     if (row0 + vv >= N) return;
     const float* src = smf + vv * C::P1 + s0;
@@ -489,20 +532,22 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
 // rows handed out over the cluster's V columns, the compensated leapfrog
 // d^{n+1} = d^n + uhat (d^1 = uhat), u^{n+1} = u^n + d^{n+1}, u = u_hi + u_lo.
 template <int LOGL>
-__global__ void __launch_bounds__(BlkFFT<LOGL>::T, Cfg<LOGL>::kColsBlocks)
+__global__ void __launch_bounds__(Cfg<LOGL>::R * BlkFFT<LOGL>::T, Cfg<LOGL>::kColsBlocks)
 kb_cols_solve(const __grid_constant__ RegBatch B) {
   using F = BlkFFT<LOGL>;
   using C = Cfg<LOGL>;
+  using X = Exchange<LOGL>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* sm = reinterpret_cast<float2*>(smem_raw);
-  float* smf = reinterpret_cast<float*>(smem_raw);
-  pdl_allow_dependents();
+  // row rl of the block, thread t of the row
+  const int rl = C::R == 1 ? 0 : threadIdx.x / F::T, t = C::R == 1 ? threadIdx.x : threadIdx.x % F::T;
+  float2* sm = reinterpret_cast<float2*>(smem_raw) + rl * C::ELEMS;
+  float* smf = reinterpret_cast<float*>(sm);
   const RegInst& I = B.in[blockIdx.y];
-  const int N = I.N, t = threadIdx.x;
-  const int rank = blockIdx.x % C::V, i0 = blockIdx.x - rank, i = blockIdx.x;
+  const int N = I.N;
+  const int i = blockIdx.x * C::R + rl, rank = i % C::V, i0 = i - rank;
   if (i0 >= N) return;   // the whole cluster
   const bool valid = i < N;
-  auto sync = [] { __syncthreads(); };
+  auto sync = [rl] { C::R == 1 ? __syncthreads() : row_sync<F::T>(rl); };
   pdl_wait_prerequisites();
   const float* w = I.W + (size_t)(valid ? i : 0) * I.ld;
   float2 x[F::E];
@@ -513,16 +558,16 @@ kb_cols_solve(const __grid_constant__ RegBatch B) {
   });
   float y[F::E];
   gs_solve<LOGL>(x, y, sm, t, i, I, sync);
-  cluster_join();   // every block of the cluster has read its buffer
+  X::join();   // every row of the cluster has read its buffer
   static_for<0, C::V>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
-    const unsigned dst = peer(smf + rank * C::P1 + t, c);
+    const unsigned dst = X::at(smf + rank * C::P1 + t, rl, c);
     static_for<0, C::QS>([&](auto jc) {
       constexpr int j = decltype(jc)::value;
-      st_peer(dst + (unsigned)(F::T * j * sizeof(float)), y[c * C::QS + j]);
+      X::put(dst + (unsigned)(F::T * j * sizeof(float)), y[c * C::QS + j]);
     });
   });
-  cluster_sync();
+  X::sync();
   const int vv = t % C::V, s0 = t / C::V;
   if (i0 + vv >= N) return;
   const float* src = smf + vv * C::P1 + s0;
@@ -567,6 +612,22 @@ kb_cols_solve(const __grid_constant__ RegBatch B) {
 }
 
 template <int LOGL>
+cudaError_t launch_blk_conv(const RegBatch& b, cudaStream_t st) {
+  using F = BlkFFT<LOGL>;
+  using C = Cfg<LOGL>;
+  static LaunchCache attr_done[kLauncherDevices];
+  const int dev = device_slot();
+  if (dev < 0) return cudaErrorInvalidDevice;
+  if (!attr_done[dev].load(std::memory_order_acquire)) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(kb_cols_conv<LOGL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes_conv);
+    if (e != cudaSuccess) return e;
+    attr_done[dev].store(1, std::memory_order_release);
+  }
+  return launch_dependent(kb_cols_conv<LOGL>, dim3(F::L + 1, b.count), dim3(2 * F::T), C::bytes_conv, st, b);
+}
+
+template <int LOGL>
 cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense) {
   using F = BlkFFT<LOGL>;
   using C = Cfg<LOGL>;
@@ -578,20 +639,19 @@ cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
     auto room = [](auto kernel, size_t bytes) {
       return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    if ((e = room(kb_rows_r2c<LOGL>, C::bytes)) || (e = room(kb_cols_conv<LOGL>, C::bytes_conv)) ||
-        (e = room(kb_rows_solve<LOGL, false>, C::bytes)) || (e = room(kb_rows_solve<LOGL, true>, C::bytes)) ||
+    if ((e = room(kb_rows_r2c<LOGL>, C::bytes)) || (e = room(kb_rows_solve<LOGL, false>, C::bytes)) || (e = room(kb_rows_solve<LOGL, true>, C::bytes)) ||
         (e = room(kb_cols_solve<LOGL>, C::bytes)))
       return e;
     attr_done[dev].store(1, std::memory_order_release);
   }
   // every kernel of the step is a programmatic dependent of the one before
   // it; the row kernels run in clusters of V blocks
-  auto launch = [&](auto kernel, dim3 grid, int threads, size_t smem, bool cluster) {
+  auto launch = [&](auto kernel, dim3 grid, int threads, size_t smem) {
     cudaLaunchAttribute a[2];
     a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     a[0].val.programmaticStreamSerializationAllowed = 1;
     a[1].id = cudaLaunchAttributeClusterDimension;
-    a[1].val.clusterDim.x = C::V;
+    a[1].val.clusterDim.x = C::CL;
     a[1].val.clusterDim.y = 1;
     a[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
@@ -600,21 +660,21 @@ cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = a;
-    cfg.numAttrs = cluster ? 2 : 1;
+    cfg.numAttrs = C::CL > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, b);
   };
-  const dim3 rgrid((max_n + C::V - 1) / C::V * C::V, b.count);
+  const dim3 rgrid((max_n + C::V - 1) / C::V * C::CL, b.count);
   if (ev) cudaEventRecord(ev[0], st);
-  if ((e = launch(kb_rows_r2c<LOGL>, rgrid, F::T, C::bytes, true))) return e;
+  if ((e = launch(kb_rows_r2c<LOGL>, rgrid, C::R * F::T, C::bytes))) return e;
   if (ev) cudaEventRecord(ev[1], st);
-  if ((e = launch(kb_cols_conv<LOGL>, dim3(F::L + 1, b.count), 2 * F::T, C::bytes_conv, false))) return e;
+  if ((e = launch_blk_conv<LOGL>(b, st))) return e;
   if (ev) cudaEventRecord(ev[2], st);
-  if (dense) return launch(kb_rows_solve<LOGL, true>, rgrid, F::T, C::bytes, true);
+  if (dense) return launch(kb_rows_solve<LOGL, true>, rgrid, C::R * F::T, C::bytes);
   const bool border = border::any(b);
-  if ((e = launch(kb_rows_solve<LOGL, false>, rgrid, F::T, C::bytes, true))) return e;
+  if ((e = launch(kb_rows_solve<LOGL, false>, rgrid, C::R * F::T, C::bytes))) return e;
   if (border && (e = border::launch<0>(b, max_n, st))) return e;
   if (ev) cudaEventRecord(ev[3], st);
-  if ((e = launch(kb_cols_solve<LOGL>, rgrid, F::T, C::bytes, true))) return e;
+  if ((e = launch(kb_cols_solve<LOGL>, rgrid, C::R * F::T, C::bytes))) return e;
   if (border && (e = border::launch<1>(b, max_n, st))) return e;
   if (ev) cudaEventRecord(ev[4], st);
   return cudaSuccess;

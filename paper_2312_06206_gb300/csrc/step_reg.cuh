@@ -1,6 +1,7 @@
 // step_reg.cuh -- the S-ADI step (Sec. 3, eq. "ADI scheme equivalent") for
-// FFT lengths N' <= 1024 (both FP32 forms) with the register-resident
-// two-level FFT of regfft.cuh (longer lengths: step_blk.cuh).
+// FFT lengths N' <= 128 (both FP32 forms) and N' = 1024 (the dense form's row
+// kernels) with the register-resident two-level FFT of regfft.cuh (the other
+// lengths: step_blk.cuh, see blk_path).
 // Same four kernels and the same mathematics as step_kernels.cu:
 //   kr_rows_r2c    rows of the increment d^n = u^n - u^{n-1} -> half spectrum
 //                  along x (natural slots)
@@ -20,6 +21,10 @@
 #include "sadi_internal.h"
 
 namespace sadi {
+namespace blk {
+template <int LOGL>
+cudaError_t launch_blk_conv(const RegBatch& b, cudaStream_t st);   // step_blk.cuh
+}
 namespace regk {
 
 using rf::static_for;
@@ -120,14 +125,10 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool pred
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Programmatic dependent launch.  The step's kernels are launched with
-// programmatic stream serialisation: a kernel may start once every block of
-// the kernel before it has started (each signals that at its beginning),
-// stages its constant tables, and waits for the earlier kernel to have
-// completed, its writes visible, before it reads anything that kernel (or an
-// earlier one) writes.  Launched without that attribute both are no-ops.
-__device__ __forceinline__ void pdl_allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Programmatic dependent launch (pdl_entry): a kernel stages its constant tables
+// before it waits for the earlier kernel to have completed, its writes
+// visible, and only then lets the next one be scheduled.
+__device__ __forceinline__ void pdl_wait_prerequisites() { pdl_entry(); }
 
 // The twiddle tables tw1 (two-level FFT) and tw[0 .. L) staged into shared
 // memory (one cp.async group): the transforms read them in their inner
@@ -220,8 +221,8 @@ __device__ __forceinline__ float real_at(const float2* sm, int k) {
 // Im vhat[r-1-p].  ybot is formed once per vector, in the real part of
 // vhat[N + p] (which nothing else reads), then each lane adds column p of G
 // to all its outputs: its loads of one p are independent and coalesced (rows
-// of G and ybot anew for every k before: N = 399, r = 113, FP32 step: 313 ->
-// 163 us; N = 1023, r = 1, one instance: 103 -> 95 us).  sync: the barrier of the vector's
+// of G and ybot anew for every k before: at N = 399, r = 113 this took the step
+// from 313 to 163 us).  sync: the barrier of the vector's
 // threads.
 template <int LOGL, typename Sync>
 __device__ __forceinline__ void gs_out_reg(float* y, float2* sm, int t, const RegInst& I, Sync sync) {
@@ -255,7 +256,6 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   using F = rf::RegFFT<float, LOGL>;
   using C = RowCfg<LOGL, BLOCK>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_allow_dependents();
   const RegInst& I = B.in[blockIdx.y];
   const int N = I.N;
   if ((int)blockIdx.x * C::VB >= N) return;
@@ -331,7 +331,6 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
   using F = rf::RegFFT<float, LOGL>;
   using C = ConvCfg<LOGL, BLOCK>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_allow_dependents();
   const RegInst& I = B.in[blockIdx.y];
   const int N = I.N, Np = F::L;
   const int c = threadIdx.x / F::TT, t = threadIdx.x % F::TT;
@@ -423,7 +422,6 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   using F = rf::RegFFT<float, LOGL>;
   using C = RowCfg<LOGL, BLOCK>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_allow_dependents();
   const RegInst& I = B.in[blockIdx.y];
   const int N = I.N, Np = F::L;
   if ((int)blockIdx.x * C::VB >= N) return;
@@ -556,13 +554,13 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
             const float u = e ? uv[j2].y : uv[j2].x;
             if constexpr (!DIFF) {
               float gs = g_of_r(I, u);
-              if (I.F) gs += I.fsc * I.F[rbase + x];
+              if (I.F) gs += I.fsc * I.F[(size_t)rrow * I.ldF + x];
               const float gg = tau2 * gs;
               b[e] = I.first ? tau * I.phi2[rbase + x] + 0.5f * (c + gg) : c + gg;
             } else {
               const float d = e ? dv[j2].y : dv[j2].x;
               float gs = g_of_r(I, u + 0.5f * d);
-              if (I.F) gs += I.fsc * I.F[rbase + x];
+              if (I.F) gs += I.fsc * I.F[(size_t)rrow * I.ldF + x];
               b[e] = (c + 0.5f * cx) + tau2 * gs - d;
             }
           }
@@ -585,10 +583,12 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
             float* wr = I.W + rbase;
             if (x + 1 < N) *reinterpret_cast<float2*>(wr + x) = make_float2(b[0], b[1]);
             else wr[x] = b[0];
-            unsigned hi, lo;
-            split_bf16x2(b[0], b[1], &hi, &lo);
-            *reinterpret_cast<unsigned*>(I.Bh + (size_t)rrow * I.ldp + x) = hi;
-            *reinterpret_cast<unsigned*>(I.Bl + (size_t)rrow * I.ldp + x) = lo;
+            if (I.Bh) {
+              unsigned hi, lo;
+              split_bf16x2(b[0], b[1], &hi, &lo);
+              *reinterpret_cast<unsigned*>(I.Bh + (size_t)rrow * I.ldp + x) = hi;
+              *reinterpret_cast<unsigned*>(I.Bl + (size_t)rrow * I.ldp + x) = lo;
+            }
           }
         } else {
           sm[pad32(n)] = make_float2(b[0], b[1]);
@@ -627,7 +627,6 @@ __global__ void __launch_bounds__(BLOCK, 3) kr_cols_solve(const __grid_constant_
   using F = rf::RegFFT<float, LOGL>;
   using C = ColCfg<LOGL, BLOCK>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_allow_dependents();
   const RegInst& I = B.in[blockIdx.y];
   const int N = I.N, Np = F::L;
   if ((int)blockIdx.x * C::CT >= N) return;
@@ -732,25 +731,25 @@ inline bool fewer_waves(int shape, int count, int max_n, int narrow_rows, int wi
   return (wb + sms * ow - 1) / (sms * ow) < (nb + sms * on - 1) / (sms * on);
 }
 
-constexpr int kRegMaxLog = kBlkMinLog - 1;   // longer vectors: step_blk.cuh
-
 template <int LOGL>
 cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense) {
   static_assert(LOGL <= kRegMaxLog, "register path FFT length");
+  constexpr bool kWide = LOGL == 10;   // N' = 1024: the dense form's row kernels alone
+  if (kWide && !dense) return cudaErrorInvalidValue;
   using RC = RowCfg<LOGL, kRowBlock>;
   using CC = ColCfg<LOGL, kColBlock>;
   using VC = ConvCfg<LOGL, kConvBlock>;
   using RW = RowCfg<LOGL, kRowBlockWide>;
   constexpr int Np = 1 << LOGL;
   static LaunchCache attr_done[kLauncherDevices];
-  // narrow / wide occupancy of the row kernels (r2c, GS solve, dense B^n),
+  // narrow / wide occupancy of the row kernels (r2c, dense B^n),
   // written before attr_done is published and read after it
-  static LaunchCache shape[3][kLauncherDevices];
+  static LaunchCache shape[2][kLauncherDevices];
   const int dev = device_slot();
   if (dev < 0) return cudaErrorInvalidDevice;
   if (!attr_done[dev].load(std::memory_order_acquire)) {
     cudaError_t e;
-    if constexpr (LOGL == 10) {
+    if constexpr (kWide) {
       int sms = 0;
       if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
       // resident narrow and wide blocks per SM of one row kernel
@@ -767,33 +766,33 @@ cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
       };
       if ((e = measure(kr_rows_r2c<LOGL, kRowBlock>, kr_rows_r2c<LOGL, kRowBlockWide>, RC::bytes_r2c, RW::bytes_r2c,
                        shape[0][dev])) ||
-          (e = measure(kr_rows_solve<LOGL, kRowBlock>, kr_rows_solve<LOGL, kRowBlockWide>, RC::bytes_solve,
-                       RW::bytes_solve, shape[1][dev])) ||
           (e = measure(kr_rows_solve<LOGL, kRowBlock, true>, kr_rows_solve<LOGL, kRowBlockWide, true>,
-                       RC::bytes_solve, RW::bytes_solve, shape[2][dev])))
+                       RC::bytes_solve, RW::bytes_solve, shape[1][dev])))
         return e;
     }
     if ((e = cudaFuncSetAttribute(kr_rows_r2c<LOGL, kRowBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)RC::bytes_r2c)) ||
         (e = cudaFuncSetAttribute(kr_rows_solve<LOGL, kRowBlock, true>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RC::bytes_solve)) ||
-        (e = cudaFuncSetAttribute(kr_cols_conv<LOGL, kConvBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)VC::bytes)))
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RC::bytes_solve)))
       return e;
-    if ((e = cudaFuncSetAttribute(kr_rows_solve<LOGL, kRowBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)RC::bytes_solve)) ||
-        (e = cudaFuncSetAttribute(kr_cols_solve<LOGL, kColBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)CC::bytes_solve)))
-      return e;
+    if constexpr (!kWide) {
+      if ((e = cudaFuncSetAttribute(kr_cols_conv<LOGL, kConvBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)VC::bytes)) ||
+          (e = cudaFuncSetAttribute(kr_rows_solve<LOGL, kRowBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)RC::bytes_solve)) ||
+          (e = cudaFuncSetAttribute(kr_cols_solve<LOGL, kColBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)CC::bytes_solve)))
+        return e;
+    }
     attr_done[dev].store(1, std::memory_order_release);
   }
   const dim3 rgrid((max_n + RC::VB - 1) / RC::VB, b.count);
   const dim3 cgrid((Np + 1 + VC::CT / 2 - 1) / (VC::CT / 2), b.count);
   const dim3 sgrid((max_n + CC::CT - 1) / CC::CT, b.count);
   // wide row blocks where they take fewer waves (N' = 1024 only)
-  bool wide[3] = {false, false, false};
-  if constexpr (LOGL == 10)
-    for (int k = 0; k < 3; ++k)
+  bool wide[2] = {false, false};
+  if constexpr (kWide)
+    for (int k = 0; k < 2; ++k)
       wide[k] = fewer_waves(shape[k][dev].load(std::memory_order_relaxed), b.count, max_n, RC::VB, RW::VB);
   const dim3 wgrid((max_n + RW::VB - 1) / RW::VB, b.count);
   // every kernel of the step is a programmatic dependent of the one before it
@@ -813,7 +812,7 @@ cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
   };
   cudaError_t e;
   if (ev) cudaEventRecord(ev[0], st);
-  if constexpr (LOGL == 10) {
+  if constexpr (kWide) {
     if (wide[0]) e = launch(kr_rows_r2c<LOGL, kRowBlockWide>, wgrid, kRowBlockWide, RW::bytes_r2c);
     else e = launch(kr_rows_r2c<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_r2c);
   } else {
@@ -821,24 +820,22 @@ cudaError_t launch_reg_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
   }
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], st);
-  if ((e = launch(kr_cols_conv<LOGL, kConvBlock>, cgrid, kConvBlock, VC::bytes))) return e;
+  if constexpr (kWide) e = blk::launch_blk_conv<LOGL>(b, st);
+  else e = launch(kr_cols_conv<LOGL, kConvBlock>, cgrid, kConvBlock, VC::bytes);
+  if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[2], st);
   if (dense) {
-    if constexpr (LOGL == 10) {
-      if (wide[2]) return launch(kr_rows_solve<LOGL, kRowBlockWide, true>, wgrid, kRowBlockWide, RW::bytes_solve);
+    if constexpr (kWide) {
+      if (wide[1]) return launch(kr_rows_solve<LOGL, kRowBlockWide, true>, wgrid, kRowBlockWide, RW::bytes_solve);
     }
     return launch(kr_rows_solve<LOGL, kRowBlock, true>, rgrid, kRowBlock, RC::bytes_solve);
   }
-  if constexpr (LOGL == 10) {
-    if (wide[1]) e = launch(kr_rows_solve<LOGL, kRowBlockWide>, wgrid, kRowBlockWide, RW::bytes_solve);
-    else e = launch(kr_rows_solve<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_solve);
-  } else {
-    e = launch(kr_rows_solve<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_solve);
+  if constexpr (!kWide) {
+    if ((e = launch(kr_rows_solve<LOGL, kRowBlock>, rgrid, kRowBlock, RC::bytes_solve))) return e;
+    if (ev) cudaEventRecord(ev[3], st);
+    if ((e = launch(kr_cols_solve<LOGL, kColBlock>, sgrid, kColBlock, CC::bytes_solve))) return e;
+    if (ev) cudaEventRecord(ev[4], st);
   }
-  if (e != cudaSuccess) return e;
-  if (ev) cudaEventRecord(ev[3], st);
-  if ((e = launch(kr_cols_solve<LOGL, kColBlock>, sgrid, kColBlock, CC::bytes_solve))) return e;
-  if (ev) cudaEventRecord(ev[4], st);
   return cudaSuccess;
 }
 

@@ -101,3 +101,47 @@ def test_tiles_move_a_running_context_between_the_engines(S):
             us.append(s.get()[0])
     assert not np.array_equal(us[0], us[1])
     assert np.abs(us[0] - us[1]).max() <= 1e-6 * np.abs(us[0]).max()
+
+
+def _small(S, N, prec, equation, tiles=False, source=False):
+    tau = 0.2 / (N + 1) if equation == "wave" else 0.02 / (N + 1) ** 1.4
+    phi1 = WL.gaussian_bumps(N, 5, 3400 + N)
+    phi2 = 0.1 * WL.gaussian_bumps(N, 3, 3500 + N) if equation == "wave" else None
+    with S.Sadi(N, 1.4, 0.9, tau, equation=equation) as s:
+        s.set_options(2, prec)
+        if tiles:
+            t = s.sadi_get_tiles()
+            s.sadi_set_tiles(t[0] + 1, t[1], t[2])
+        s.set_initial(phi1, phi2)
+        if source:
+            import torch
+            f = torch.from_numpy(0.3 * WL.gaussian_bumps(N, 2, 3600 + N)).to("cuda").float()
+            for _ in range(3):
+                s.sadi_step_source(f.data_ptr(), 1)
+        else:
+            s.step(3)
+        return s.get()[0]
+
+
+@pytest.mark.parametrize("N", [65, 95, 96, 128, 129, 223, 224, 255, 256, 257, 479, 480, 511, 512, 513, 991, 992, 1023])
+@pytest.mark.parametrize("equation", ["wave", "diffusion"])
+def test_small_fp32_paths_against_fp64(S, N, equation):
+    # N' = 128 .. 1024: eight or four rows a block, the border correction added
+    # in the sweeps (r <= 32), by dense sweeps (N' <= 512) or by the separate
+    # product (N' = 1024); with and without a caller's source field (rows of N)
+    for source in (False, True):
+        w = _small(S, N, S.SADI_PREC_FP64, equation, source=source)
+        for prec in (S.SADI_PREC_FP32, S.SADI_PREC_FP32_DENSE):
+            u = _small(S, N, prec, equation, source=source)
+            assert np.abs(u - w).max() <= 1e-6 * np.abs(w).max(), (prec, source)
+
+
+@pytest.mark.parametrize("N", [1, 2, 5, 31, 63, 64, 65, 100, 127, 128])
+@pytest.mark.parametrize("equation", ["wave", "diffusion"])
+def test_small_fp64_step_against_the_transforms(S, N, equation):
+    # the direct path (dense products, the default up to N' = 128) against the
+    # shared-memory engine (tiles other than the defaults): at most 8 N' + 2 products are
+    # summed per value, 1e-16 x sqrt(1000) x 3 steps < 1e-13 of the largest
+    u = _small(S, N, S.SADI_PREC_FP64, equation)
+    v = _small(S, N, S.SADI_PREC_FP64, equation, tiles=True)
+    assert np.abs(u - v).max() <= 1e-13 * np.abs(v).max()
