@@ -1,7 +1,7 @@
 // step_blk.cuh -- the FP32 S-ADI step (Sec. 3, eq. "ADI scheme equivalent")
-// for FFT lengths N' = 2048 .. 8192 on the block-wide register FFT of
-// blkfft.cuh.  The four kernels of step_reg.cuh, with one row, column half or
-// column per T = 128 or 256 threads:
+// for FFT lengths N' = 256 .. 8192 (blk_path) on the block-wide register FFT
+// of blkfft.cuh.  The four kernels of step_reg.cuh, with one row, column half
+// or column per T = 32 .. 256 threads:
 //   kb_rows_r2c    row of the increment d^n -> half spectrum along x
 //   kb_cols_conv   x frequency: y FFT (even / odd half) x symbol, inverse
 //   kb_rows_solve  inverse real FFT, C += conv(d^n), B^n, then the x sweep
@@ -12,17 +12,17 @@
 // the spectrum is stored by x frequency (S[k * lds + row]) and the x sweep's
 // result by column (W[k * ld + row]), so that each column kernel reads one
 // contiguous vector.  A single row would then move 8- or 4-byte pieces a
-// column apart; the rows of a cluster of V = 8 blocks are therefore exchanged
-// through distributed shared memory: block c of the cluster gathers
-// frequencies (columns) c L/V .. of all V rows and moves runs of V rows, 64 or
-// 32 bytes.  This replaces the two transpose passes of the shared-memory
+// column apart; groups of V = 8 rows, in one block (R = 8) or in a cluster of
+// V / R, are therefore exchanged through (distributed) shared memory: row c of
+// the group gathers frequencies (columns) c L/V .. of all V rows and moves runs
+// of V rows, 64 or 32 bytes.  This replaces the two transpose passes of the shared-memory
 // engine's y sweep and its 8-byte column gathers.
 //
 // Measured against the shared-memory engine (us per launch, GB300): N = 4095
-// row FFT 145 -> 94, convolution 407 -> 193, B^n 258 -> 177, GS rows 537 ->
-// 365, y sweep 488 (with its transposes) -> 290; N = 8191 row FFT 681 -> 418,
-// convolution 1822 (three passes) -> 1103, GS rows 2649 -> 1921, y sweep 2241
-// -> 1263; N = 2047, four instances: 80 + 192 + 264 -> 75 + 175 + 170 against
+// row FFT 145 -> 93, convolution 407 -> 157, B^n 258 -> 177, GS rows 537 ->
+// 370, y sweep 488 (with its transposes) -> 292; N = 8191 row FFT 681 -> 415,
+// convolution 1822 (three passes) -> 737, GS rows 2649 -> 1750, y sweep 2241
+// -> 1260; N = 2047, four instances: 80 + 192 + 264 -> 75 + 175 + 170 against
 // the 64-elements-per-lane kernels this replaces there.  Instructions per
 // element and transform fell from 134 to about 50; what bounds the kernels now
 // is the latency of the table loads and barriers at 16 to 32 warps per SM
@@ -121,19 +121,23 @@ struct Cfg {
   static constexpr int ELEMS = F::BUF > V * P2 ? F::BUF : V * P2;
   static_assert(V * P1 <= 2 * ELEMS, "the float exchange buffer fits too");
   static constexpr size_t bytes = (size_t)R * ELEMS * sizeof(float2);
-  static constexpr size_t bytes_conv = 2 * (size_t)F::BUF * sizeof(float2);
+  static constexpr size_t bytes_conv = (size_t)(F::BUF + (LOGL <= 10 ? F::BUF : F::L)) * sizeof(float2);
   // resident blocks promised to the compiler (its register budget), measured
   // at N = 4095 (us per launch at 2 / 3 / 4 blocks of 256 threads): r2c 109 /
-  // 100 / 94, dense B^n 208 / 179 / 177, GS rows 378 / 362 / -, columns
-  // 289 / 312, convolution 193 (one block of 512 threads, 128 registers)
-  // against 219 (two, 64 registers).  E = 32 (N' = 8192) needs 128 registers.
+  // 100 / 94, dense B^n 208 / 179 / 177, GS rows 378 / 362 / -, columns 289 /
+  // 312.  E = 32 (N' = 8192) needs 128 registers.  Seven N = 511 instances,
+  // dense B^n: 18 us at 64 registers, 21 at 85.
   static constexpr int kM = 256 / F::T;   // rows for each 256 threads
   static constexpr int per(int rows) { return rows / R > 0 ? rows / R : 1; }
   static constexpr int kR2cBlocks = per(LOGL == 13 ? 2 : 4 * kM);
-  static constexpr int kDenseBlocks = per(LOGL == 13 ? 2 : LOGL >= 11 ? 4 * kM : 2 * kM);
+  static constexpr int kDenseBlocks = per(LOGL == 13 ? 2 : LOGL >= 11 ? 4 * kM : LOGL == 9 ? 4 * kM : 2 * kM);
   static constexpr int kGsBlocks = per(LOGL == 13 ? 2 : LOGL >= 11 ? 3 * kM : 2 * kM);
   static constexpr int kColsBlocks = per(2 * kM);
-  static constexpr int kConvBlocks = LOGL >= 11 ? kM : F::E == 8 ? 2 * kM : kM;
+  // the two convolution kernels: both halves in one block up to N' = 1024
+  // (29 us at 4 blocks a SM, 30 at 5, 31 at 6 for three N = 1023 instances),
+  // one after the other above
+  static constexpr bool kConvSplit = LOGL <= 10;
+  static constexpr int kConvBlocks = LOGL == 10 ? 4 : LOGL == 9 ? 6 : LOGL == 8 ? 12 : LOGL == 13 ? 1 : 2 * kM;
 };
 
 // Exchange between the V rows of a cluster: barriers over all of them and the
@@ -286,6 +290,65 @@ kb_cols_conv(const __grid_constant__ RegBatch B) {
     constexpr int q = decltype(qc)::value;
     const int j = t + F::T * (h ? q + HE : q);
     const float2 y = cadd(h ? x[q + HE] : x[q], other[F::T * q]);
+    if (j < N) {
+      if (kx == 0) reinterpret_cast<float*>(col + j)[0] = y.x;
+      else if (kx == F::L) reinterpret_cast<float*>(col + j)[1] = y.x;
+      else col[j] = y;
+    }
+  });
+}
+
+// The same with one half after the other on T threads, from N' = 2048 on: the
+// even half's result waits in shared memory (each thread its own elements),
+// and the odd half reads the column again (from L2).  Independent blocks with
+// their full registers overlap loads, transforms and stores, where the split
+// kernel's one block of 512 threads an SM ran in lockstep (N = 4095 193 -> 157
+// us, N = 8191, 255 registers and no spills, 1098 -> 737); more blocks than two
+// an SM take L1 from the tables and lose (174 at three, 205 at four).
+template <int LOGL>
+__global__ void __launch_bounds__(BlkFFT<LOGL>::T, Cfg<LOGL>::kConvBlocks)
+kb_cols_conv_seq(const __grid_constant__ RegBatch B) {
+  using F = BlkFFT<LOGL>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const RegInst& I = B.in[blockIdx.y];
+  const int N = I.N, kx = blockIdx.x, t = threadIdx.x;
+  float2* const sm = reinterpret_cast<float2*>(smem_raw);
+  float2* const keep = sm + F::BUF + t;
+  auto sync = [] { __syncthreads(); };
+  float2* col = I.S + (size_t)(kx == F::L ? 0 : kx) * I.lds;
+  pdl_wait_prerequisites();
+  float2 x[F::E];
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    if (kx == 0 || kx == F::L) {
+      const float* c1 = reinterpret_cast<const float*>(col) + (kx == 0 ? 0 : 1);
+      static_for<0, F::E>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        const int j = t + F::T * q;
+        x[q] = make_float2(j < N ? c1[2 * j] : 0.f, 0.f);
+      });
+    } else {
+      static_for<0, F::E>([&](auto qc) {
+        constexpr int q = decltype(qc)::value;
+        const int j = t + F::T * q;
+        x[q] = j < N ? col[j] : make_float2(0.f, 0.f);
+      });
+    }
+    const float2* tw1 = h ? I.btw1h : I.btw1;
+    F::fwd(x, sm, t, tw1, h, I.btw2, sync);
+    const float* lam = I.lnat + (size_t)kx * (F::L + 1);
+    static_for<0, F::E>([&](auto qc) {
+      constexpr int q = decltype(qc)::value;
+      const int k2 = 2 * (t + F::T * q) + h;
+      x[q] = cscale(x[q], __ldg(&lam[q < F::E / 2 ? k2 : 2 * F::L - k2]));
+    });
+    F::inv(x, sm, t, tw1, h, I.btw2, sync);
+    if (h == 0) static_for<0, F::E>([&](auto qc) { keep[F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
+  }
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int j = t + F::T * q;
+    const float2 y = cadd(keep[F::T * q], x[q]);
     if (j < N) {
       if (kx == 0) reinterpret_cast<float*>(col + j)[0] = y.x;
       else if (kx == F::L) reinterpret_cast<float*>(col + j)[1] = y.x;
@@ -618,13 +681,17 @@ cudaError_t launch_blk_conv(const RegBatch& b, cudaStream_t st) {
   static LaunchCache attr_done[kLauncherDevices];
   const int dev = device_slot();
   if (dev < 0) return cudaErrorInvalidDevice;
-  if (!attr_done[dev].load(std::memory_order_acquire)) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(kb_cols_conv<LOGL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes_conv);
-    if (e != cudaSuccess) return e;
-    attr_done[dev].store(1, std::memory_order_release);
-  }
-  return launch_dependent(kb_cols_conv<LOGL>, dim3(F::L + 1, b.count), dim3(2 * F::T), C::bytes_conv, st, b);
+  auto go = [&](auto kernel, int threads) {
+    if (!attr_done[dev].load(std::memory_order_acquire)) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes_conv);
+      if (e != cudaSuccess) return e;
+      attr_done[dev].store(1, std::memory_order_release);
+    }
+    return launch_dependent(kernel, dim3(F::L + 1, b.count), dim3(threads), C::bytes_conv, st, b);
+  };
+  if constexpr (C::kConvSplit) return go(kb_cols_conv<LOGL>, 2 * F::T);
+  else return go(kb_cols_conv_seq<LOGL>, F::T);
 }
 
 template <int LOGL>
