@@ -1381,10 +1381,12 @@ extern "C" sadi_status sadi_step_source(sadi_ctx* c, const void* f, int dtype) {
   const bool f64 = c->prec == SADI_PREC_FP64;
   const int N = c->g.N, ld = c->g.ld;
   const void* field = f;
-  // the caller's field is used in place when its type is the context's and the
-  // step's kernels take its row pitch (the register paths take any); else it
-  // is converted (and its rows spread to the padded pitch)
-  if ((dtype == 0) != f64 || (ld != N && !c->reg_path)) {
+  // the caller's field is used in place when its type is the context's, the
+  // step's kernels take its row pitch (the register paths take any) and its
+  // elements are aligned; else it is converted (and its rows spread to the
+  // padded pitch)
+  const bool aligned = reinterpret_cast<uintptr_t>(f) % (f64 ? sizeof(double) : sizeof(float)) == 0;
+  if ((dtype == 0) != f64 || (ld != N && !(c->reg_path && aligned))) {
     if (!c->Fconv) CK(cudaMalloc(&c->Fconv, (size_t)ld * N * esize(c->prec)), "cudaMalloc(source conversion)");
     if (f64)
       CK(launch_convert_f2d(static_cast<const float*>(f), static_cast<double*>(c->Fconv), N, N, N, ld, c->stream),

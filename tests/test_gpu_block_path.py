@@ -145,3 +145,23 @@ def test_small_fp64_step_against_the_transforms(S, N, equation):
     u = _small(S, N, S.SADI_PREC_FP64, equation)
     v = _small(S, N, S.SADI_PREC_FP64, equation, tiles=True)
     assert np.abs(u - v).max() <= 1e-13 * np.abs(v).max()
+
+
+@pytest.mark.parametrize("N", [100, 300, 1023])
+def test_source_field_off_its_alignment_is_copied(S, N):
+    # a float field at an odd address is copied before the step reads it; the
+    # same field on its alignment is read in place: the same bits
+    import torch
+    f = torch.from_numpy(0.3 * WL.gaussian_bumps(N, 2, 3700 + N)).to("cuda").float()
+    buf = torch.zeros(4 * N * N + 16, dtype=torch.uint8, device="cuda")
+    buf[2:2 + 4 * N * N] = f.reshape(-1).view(torch.uint8)
+    torch.cuda.synchronize()
+    out = []
+    for p in (f.data_ptr(), buf.data_ptr() + 2):
+        with S.Sadi(N, 1.4, 0.9, 0.2 / (N + 1)) as s:
+            s.set_options(1, S.SADI_PREC_FP32)
+            s.set_initial(WL.gaussian_bumps(N, 4, 3800 + N))
+            for _ in range(2):
+                s.sadi_step_source(p, 1)
+            out.append(s.get()[0])
+    assert np.array_equal(out[0], out[1])
