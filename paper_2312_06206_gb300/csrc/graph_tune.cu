@@ -262,9 +262,7 @@ sadi_status sadi_autotune(sadi_ctx** ctxs, int count, int g, int flags) {
       if (st != SADI_OK) return st;
       double ms = 0;
       if ((st = time_group(grp, 5, &ms)) != SADI_OK) return st;
-      // the shared-memory engine's decompositions beside the register path,
-      // where the GS form may run on either (explicit tiles)
-      if (prec == SADI_PREC_FP32 && logNp >= kTilesMinLog) {
+      if (!reg_path_supported(logNp, prec)) {
         // coordinate descent over the shared-memory engine's decomposition;
         // the column convolution may also run as three passes (kConvThreePass)
         Tiles t = grp[0]->tiles32;

@@ -197,7 +197,8 @@ struct RegBatch {
   RegInst in[kMaxBatch];
 };
 // FFT lengths of the two register paths: step_reg.cuh (a row per part of a warp)
-// up to 2^kRegMaxLog, step_blk.cuh (a row per warp or more) from 2^kBlkMinLog;
+// up to 2^kRegMaxLog, step_blk.cuh (a row per warp or more) from 2^kBlkMinLog
+// (reg_path_supported: to 1024 in the GS form, 2048 in the dense form);
 // explicit tiles select the shared-memory engine from 2^kTilesMinLog on.
 constexpr int kRegMaxLog = 10, kBlkMinLog = 8, kTilesMinLog = 11;
 // whether step_blk.cuh serves a context, else step_reg.cuh.  From N' = 256 on it

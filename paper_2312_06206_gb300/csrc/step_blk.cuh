@@ -1,5 +1,5 @@
 // step_blk.cuh -- the FP32 S-ADI step (Sec. 3, eq. "ADI scheme equivalent")
-// for FFT lengths N' = 256 .. 8192 (blk_path) on the block-wide register FFT
+// for FFT lengths N' = 256 .. 2048 (blk_path) on the block-wide register FFT
 // of blkfft.cuh.  The four kernels of step_reg.cuh, with one row, column half
 // or column per T = 32 .. 256 threads:
 //   kb_rows_r2c    row of the increment d^n -> half spectrum along x

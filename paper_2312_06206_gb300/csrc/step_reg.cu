@@ -12,9 +12,15 @@ template <int LOGL>
 cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaEvent_t* ev, bool dense);
 }  // namespace blk
 
-// both FP32 forms at every FFT length
+// GS form up to N' = 1024, dense form up to 2048.  Above, the block-wide FFT
+// was faster (N = 4095 GS step 0.91 ms against 1.56) but less exact: after 1000
+// steps the GS form was 1.06e-6 from FP64 at N = 2047 against 4.7e-7 on the
+// shared-memory engine, 5.9e-7 against 3.1e-7 at N = 4095; the dense form 3.4e-7
+// against 1.9e-7 at N = 4095.  At the lengths kept it is the more exact one (N =
+// 1023 GS 9.9e-7 against 1.4e-6, N = 2047 dense 3.1e-7 against 4.8e-7).
 bool reg_path_supported(int logNp, int prec) {
-  return (prec == SADI_PREC_FP32 || prec == SADI_PREC_FP32_DENSE) && logNp >= 3 && logNp <= 13;
+  if (prec == SADI_PREC_FP32) return logNp >= 3 && logNp <= 10;
+  return prec == SADI_PREC_FP32_DENSE && logNp >= 3 && logNp <= 11;
 }
 
 // block: on step_blk.cuh (blk_path), else step_reg.cuh
@@ -32,8 +38,6 @@ cudaError_t launch_step_reg(const RegBatch& b, int logNp, bool block, int max_n,
     case 16 + 9: return blk::launch_blk_impl<9>(b, max_n, st, ev, dense);
     case 16 + 10: return blk::launch_blk_impl<10>(b, max_n, st, ev, dense);
     case 16 + 11: return blk::launch_blk_impl<11>(b, max_n, st, ev, dense);
-    case 16 + 12: return blk::launch_blk_impl<12>(b, max_n, st, ev, dense);
-    case 16 + 13: return blk::launch_blk_impl<13>(b, max_n, st, ev, dense);
     default: return cudaErrorInvalidValue;
   }
 }

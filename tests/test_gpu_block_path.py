@@ -50,7 +50,10 @@ def test_block_path_against_shared_memory_engine(S, N, equation, prec_name):
     prec = getattr(S, prec_name)
     u = _run(S, N, prec, equation)
     v = _run(S, N, prec, equation, tiles=True)
-    assert not np.array_equal(u, v)          # two engines, not one
+    # the block path is the default for the dense form at N' = 2048 only; else
+    # explicit tiles equal to the defaults are the same engine
+    two = prec == S.SADI_PREC_FP32_DENSE and N <= 2048
+    assert np.array_equal(u, v) != two
     assert np.abs(u - v).max() <= 1e-6 * np.abs(v).max()
     if N in (1025, 2015, 2048):
         w = _run(S, N, S.SADI_PREC_FP64, equation)
@@ -82,8 +85,8 @@ def test_block_path_batch_of_uneven_border_ranks(S):
 
 
 def test_tiles_move_a_running_context_between_the_engines(S):
-    # both engines keep the state in one layout: an FP32 context may change
-    # engine between steps
+    # tiles set and cleared between steps: the GS form at N' = 2048 has one
+    # engine, so nothing changes
     N = 1100
     phi1 = WL.gaussian_bumps(N, 4, 3300)
     us = []
@@ -99,8 +102,7 @@ def test_tiles_move_a_running_context_between_the_engines(S):
                 s.sadi_set_tiles(0, 0, 0)
             s.step(1)
             us.append(s.get()[0])
-    assert not np.array_equal(us[0], us[1])
-    assert np.abs(us[0] - us[1]).max() <= 1e-6 * np.abs(us[0]).max()
+    assert np.array_equal(us[0], us[1])
 
 
 def _small(S, N, prec, equation, tiles=False, source=False):
