@@ -412,8 +412,10 @@ def roofline_of(phase_ms, N, Np, dense, ninst, workload):
     kernel's bound is the roof its algorithmic intensity (method flops per
     method byte) meets first: HBM below the ridge FP32 peak / HBM peak, the
     FP32 pipes above it; a kernel with no method flops is HBM-bound."""
-    # the register path: both forms up to N' = 1024, the dense form's FFT part
-    # at N' = 2048 too
+    # the phases' labels, by the kernels of the shared-memory engine and of the
+    # register path up to N' = 1024 (the dense form's FFT part: 2048); the block
+    # path (kb_rows_r2c, kb_cols_conv*, kb_rows_solve, kb_cols_solve) reports
+    # its phases under the same labels
     reg = Np <= 1024 or (dense and Np == 2048)
     pre = "kr_" if reg else "k_"
     conv = "kr_cols_conv" if reg else ("k_conv3_a+b+c" if Np == 8192 else "k_cols_conv")   # three passes at 8192

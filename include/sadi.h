@@ -128,8 +128,8 @@ sadi_status sadi_set_options(sadi_ctx *ctx, int g, int prec);
 /* g(u) = c1 u + c3 u^3 + cs sin u (finite coefficients, else SADI_EINVAL):
  * selects SADI_G_GENERAL with these coefficients; the nonlinear term enters
  * B^n as the paper's g does (Sec. 3), evaluated in the step's precision (the
- * FP32 register path uses the hardware sine, whose error is scaled by
- * tau^2).  Must precede sadi_set_initial (SADI_ESTATE otherwise). */
+ * FP32 forms use the hardware sine at N' <= 128 and, FP32_DENSE, at N' = 1024;
+ * its error is scaled by tau^2).  Must precede sadi_set_initial (SADI_ESTATE otherwise). */
 sadi_status sadi_set_nonlinearity(sadi_ctx *ctx, double c1, double c3, double cs);
 
 /* Current g and precision of ctx (either pointer may be NULL). */
