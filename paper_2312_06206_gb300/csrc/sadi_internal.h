@@ -199,7 +199,8 @@ struct RegBatch {
 // FFT lengths of the two register paths: step_reg.cuh (a row per part of a warp)
 // up to 2^kRegMaxLog, step_blk.cuh (a row per warp or more) from 2^kBlkMinLog
 // (reg_path_supported: to 1024 in the GS form, 2048 in the dense form);
-// explicit tiles select the shared-memory engine from 2^kTilesMinLog on.
+// explicit tiles select the shared-memory engine from 2^kTilesMinLog on (the
+// dense form at 2048; the others run on it anyway).
 constexpr int kRegMaxLog = 10, kBlkMinLog = 8, kTilesMinLog = 11;
 // whether step_blk.cuh serves a context, else step_reg.cuh.  From N' = 256 on it
 // measured faster for one instance and for many (us per step, step_reg.cuh ->
