@@ -131,6 +131,9 @@ sadi_status build_direct(sadi_ctx* c, int mode) {
     // kappa tau^2 h^-alpha (wave) or kappa tau h^-alpha (diffusion) is 2 s
     CK(run_dir_tables(static_cast<double*>(c->dF), static_cast<double*>(c->dT), c->a2d, c->g.N, -2.0 * c->s, st),
        "direct path tables");
+    // a step may come on another stream (sadi_set_stream), and its first
+    // kernel reads the tables before its dependency wait
+    CK(cudaStreamSynchronize(st), "direct path tables");
   }
   return SADI_OK;
 }
