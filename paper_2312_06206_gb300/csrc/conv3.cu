@@ -378,7 +378,8 @@ cudaError_t conv3_setup(int Np, int logNp, const float* lpb32, Conv3* c, cudaStr
   }
   k_conv3_symbol<<<(unsigned)((nlt + 255) / 256), 256, 0, st>>>(lpb32, z, Np, logNp);
   k_conv3_twiddles<<<(Np + 255) / 256, 256, 0, st>>>(z, Np);
-  if ((e = cudaGetLastError())) {
+  // waited for: a step may come on another stream (sadi_set_stream)
+  if ((e = cudaGetLastError()) || (e = cudaStreamSynchronize(st))) {
     conv3_free(&z);
     return e;
   }

@@ -45,3 +45,15 @@ def test_precision_switched_back_to_fp64_leaves_no_pending_work(env, N):
             out.append((s.get()[0], u[2].cpu().numpy()))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+def test_three_pass_convolution_set_up_leaves_no_pending_work(env):
+    # explicit tiles with conv_cols = -1 build the symbol table of the three
+    # passes (134 MB at N' = 4096)
+    S, torch = env
+    setup = torch.cuda.Stream()
+    with S.Sadi(4090, 1.6, 1.0, 1e-4) as s:
+        s.set_stream(setup.cuda_stream)
+        s.set_options(1, S.SADI_PREC_FP32)
+        s.sadi_set_tiles(1, -1, 1)
+        assert setup.query()
