@@ -79,14 +79,6 @@ __device__ __forceinline__ void cluster_sync() {
   cluster_arrive();
   cluster_wait();
 }
-// Execution barrier of the cluster without the release fence (about 700
-// cycles): enough where only this block's own reads have to be over before
-// its peers write (the block barrier in front completes them).
-__device__ __forceinline__ void cluster_join() {
-  __syncthreads();
-  cluster_arrive_relaxed();
-  cluster_wait();
-}
 __device__ __forceinline__ void st_peer(unsigned a, float2 v) {
   asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
@@ -140,15 +132,13 @@ struct Cfg {
   static constexpr int kConvBlocks = LOGL == 10 ? 4 : LOGL == 9 ? 6 : LOGL == 8 ? 12 : LOGL == 13 ? 1 : 2 * kM;
 };
 
-// Exchange between the V rows of a cluster: barriers over all of them and the
-// address of p (in the calling row's buffer) in the buffer of row `to`.
+// Exchange between the V rows of a cluster: the barrier over all of them
+// (release / acquire: it orders a block's own reads before its peers' writes to
+// the same buffer, and the peers' writes before its reads) and the address of p
+// (in the calling row's buffer) in the buffer of row `to`.
 template <int LOGL>
 struct Exchange {
   using C = Cfg<LOGL>;
-  __device__ static __forceinline__ void join() {   // no release: see cluster_join
-    if constexpr (C::CL == 1) __syncthreads();
-    else cluster_join();
-  }
   __device__ static __forceinline__ void sync() {
     if constexpr (C::CL == 1) __syncthreads();
     else cluster_sync();
@@ -215,7 +205,7 @@ kb_rows_r2c(const __grid_constant__ RegBatch B) {
     const float2 Ov = cscale(cmul_mi(csub(Z, Zc)), 0.5f);
     x[q] = (q == 0 && t == 0) ? make_float2(Ev.x + Ov.x, Ev.x - Ov.x) : cadd(Ev, cmul(__ldg(&I.tw[k]), Ov));
   });
-  X::join();   // every row of the cluster has read its buffer
+  X::sync();   // every row of the cluster has read its buffer
   static_for<0, C::V>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
     const unsigned dst = X::at(sm + rank * C::P2 + t, rl, c);
@@ -568,7 +558,7 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
     sync();
     float y[F::E];
     gs_solve<LOGL>(x, y, sm, t, row, I, sync);
-    X::join();   // every row of the cluster has read its buffer
+    X::sync();   // every row of the cluster has read its buffer
     float* smf = reinterpret_cast<float*>(sm);
     static_for<0, C::V>([&](auto cc) {
       constexpr int c = decltype(cc)::value;
@@ -621,7 +611,7 @@ kb_cols_solve(const __grid_constant__ RegBatch B) {
   });
   float y[F::E];
   gs_solve<LOGL>(x, y, sm, t, i, I, sync);
-  X::join();   // every row of the cluster has read its buffer
+  X::sync();   // every row of the cluster has read its buffer
   static_for<0, C::V>([&](auto cc) {
     constexpr int c = decltype(cc)::value;
     const unsigned dst = X::at(smf + rank * C::P1 + t, rl, c);
