@@ -153,8 +153,9 @@ sadi_status sadi_set_source(sadi_ctx *ctx, const double *F, double omega, double
  * fused into the B^n epilogue.  f: device memory on the context's device,
  * N*N elements (layout above) of dtype 0 = double or 1 = float, owned by the
  * caller and read by the step on the context's stream (keep it unchanged
- * until the step has run).  A dtype other than the step's precision is
- * converted into a buffer of the context (allocated on first use) first.
+ * until the step has run).  A field of a dtype other than the step's
+ * precision, or off the alignment of its elements, is converted or copied
+ * into a buffer of the context (allocated on first use) first.
  * SADI_EINVAL if f is not such a buffer; SADI_ESTATE while a separable source
  * (sadi_set_source) is set or before sadi_set_initial. */
 sadi_status sadi_step_source(sadi_ctx *ctx, const void *f, int dtype);

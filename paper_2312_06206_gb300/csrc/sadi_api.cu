@@ -1386,21 +1386,27 @@ extern "C" sadi_status sadi_step_source(sadi_ctx* c, const void* f, int dtype) {
   const void* field = f;
   // the caller's field is used in place when its type is the context's, the
   // step's kernels take its row pitch (the register paths take any) and its
-  // elements are aligned; else it is converted (and its rows spread to the
-  // padded pitch)
-  const bool aligned = reinterpret_cast<uintptr_t>(f) % (f64 ? sizeof(double) : sizeof(float)) == 0;
-  if ((dtype == 0) != f64 || (ld != N && !(c->reg_path && aligned))) {
+  // elements are aligned; else it is copied or converted (and its rows spread
+  // to the padded pitch).  The copies take any address; a conversion reads a
+  // field off the alignment of its own type from an aligned copy.
+  const size_t fsize = dtype == 0 ? sizeof(double) : sizeof(float);
+  const bool aligned = reinterpret_cast<uintptr_t>(f) % fsize == 0, same = (dtype == 0) == f64;
+  if (!same || !aligned || (ld != N && !c->reg_path)) {
     if (!c->Fconv) CK(cudaMalloc(&c->Fconv, (size_t)ld * N * esize(c->prec)), "cudaMalloc(source conversion)");
-    if (f64)
+    if (!same && !aligned) {
+      CK(stage_acquire(c), "order after the last asynchronous read");
+      CK(cudaMemcpyAsync(c->stage, f, nn * fsize, cudaMemcpyDeviceToDevice, c->stream), "source copy");
+      f = c->stage;
+    }
+    if (same)
+      CK(cudaMemcpy2DAsync(c->Fconv, ld * fsize, f, N * fsize, N * fsize, N, cudaMemcpyDeviceToDevice, c->stream),
+         "source copy");
+    else if (f64)
       CK(launch_convert_f2d(static_cast<const float*>(f), static_cast<double*>(c->Fconv), N, N, N, ld, c->stream),
          "source convert");
-    else if (dtype == 0)
+    else
       CK(launch_convert_d2f(static_cast<const double*>(f), static_cast<float*>(c->Fconv), N, N, N, ld, c->stream),
          "source convert");
-    else
-      CK(cudaMemcpy2DAsync(c->Fconv, (size_t)ld * sizeof(float), f, (size_t)N * sizeof(float), (size_t)N * sizeof(float),
-                           N, cudaMemcpyDeviceToDevice, c->stream),
-         "source copy");
     field = c->Fconv;
   }
   c->F_step = field;
