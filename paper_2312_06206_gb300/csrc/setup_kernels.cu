@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include "blkfft.cuh"
+#include "ddouble.cuh"
 #include "fft.cuh"
 #include "sadi_internal.h"
 
@@ -549,6 +550,33 @@ __global__ void k_dir_inverse(const double* __restrict__ c, int n, int ld, int i
   inverse_diagonal(c, n, [&](int i, int j, double e) { E[(size_t)i * ld + j] = (T)(i == j && !ident ? e + 1.0 : e); });
 }
 
+// One step of X <- X + X (I - H X), H = I + s T(a1), for the inverse that the
+// recurrence above leaves a few units in the last place off (N = 128: 4e-15),
+// an error of the operator in every step: the residual in double-double, the
+// correction in double.  X = I + E (ident) or E.
+__global__ void k_dir_residual(const double* __restrict__ a1, int n, int ld, double s, int ident,
+                               const double* __restrict__ E, double* R) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n * n) return;
+  const int i = idx / n, j = idx % n;
+  auto h = [&](int k) { return dd::two_prod(s, a1[k < 0 ? -k : k]); };   // (s T)_{i, i+k}
+  // ident: I - H X = -(E + s T + s T E)
+  dd::D2 acc = dd::add(h(i - j), {0.0, 0.0});
+  if (!ident) acc = {i == j ? -1.0 : 0.0, 0.0};
+  acc = dd::add(acc, {E[(size_t)i * ld + j], 0.0});
+  for (int k = 0; k < n; ++k) acc = dd::add(acc, dd::mul(h(i - k), E[(size_t)k * ld + j]));
+  R[idx] = -(acc.hi + acc.lo);
+}
+__global__ void k_dir_refine(int n, int ld, int ident, const double* __restrict__ R, const double* __restrict__ E,
+                             double* out) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n * n) return;
+  const int i = idx / n, j = idx % n;
+  double d = ident ? R[idx] : 0.0;
+  for (int k = 0; k < n; ++k) d += E[(size_t)i * ld + k] * R[k * n + j];
+  out[idx] = E[(size_t)i * ld + j] + d;
+}
+
 #define SADI_TRY(x)                        \
   do {                                     \
     cudaError_t e_ = (x);                  \
@@ -692,6 +720,7 @@ cudaError_t run_dir_inverse(const double* a1, int N, int ld, double s, bool iden
   cudaError_t err = cudaSuccess;
   int* dstat = nullptr;
   double* c = nullptr;
+  [[maybe_unused]] double* R = nullptr;   // residual, refined inverse
   *status_host = 1;
   SADI_TRY(cudaFuncSetAttribute(k_durbin, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   SADI_TRY(cudaMalloc(&dstat, sizeof(int)));
@@ -700,11 +729,22 @@ cudaError_t run_dir_inverse(const double* a1, int N, int ld, double s, bool iden
   SADI_TRY(cudaGetLastError());
   k_dir_inverse<T><<<nblk(N, 32), 32, 0, st>>>(c, N, ld, ident ? 1 : 0, E);
   SADI_TRY(cudaGetLastError());
+  if constexpr (sizeof(T) == 8) {
+    const unsigned nb = nblk((size_t)N * N, 128);
+    SADI_TRY(cudaMalloc(&R, sizeof(double) * 2 * N * N));
+    k_dir_residual<<<nb, 128, 0, st>>>(a1, N, ld, s, ident ? 1 : 0, E, R);
+    SADI_TRY(cudaGetLastError());
+    k_dir_refine<<<nb, 128, 0, st>>>(N, ld, ident ? 1 : 0, R, E, R + (size_t)N * N);
+    SADI_TRY(cudaGetLastError());
+    SADI_TRY(cudaMemcpy2DAsync(E, sizeof(double) * ld, R + (size_t)N * N, sizeof(double) * N, sizeof(double) * N, N,
+                               cudaMemcpyDeviceToDevice, st));
+  }
   SADI_TRY(cudaMemcpyAsync(status_host, dstat, sizeof(int), cudaMemcpyDeviceToHost, st));
   SADI_TRY(cudaStreamSynchronize(st));
 done:
   cudaFree(dstat);
   cudaFree(c);
+  cudaFree(R);
   return err;
 }
 template cudaError_t run_dir_inverse<float>(const double*, int, int, double, bool, float*, int*, cudaStream_t);
