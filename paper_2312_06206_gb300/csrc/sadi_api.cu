@@ -1384,14 +1384,14 @@ extern "C" sadi_status sadi_step_source(sadi_ctx* c, const void* f, int dtype) {
   const bool f64 = c->prec == SADI_PREC_FP64;
   const int N = c->g.N, ld = c->g.ld;
   const void* field = f;
-  // the caller's field is used in place when its type is the context's, the
-  // step's kernels take its row pitch (the register paths take any) and its
-  // elements are aligned; else it is copied or converted (and its rows spread
-  // to the padded pitch).  The copies take any address; a conversion reads a
-  // field off the alignment of its own type from an aligned copy.
+  // the caller's field, rows of N, is used in place when its type is the
+  // context's and its elements are aligned; else it is copied or converted (and
+  // its rows spread to the padded pitch).  The copies take any address; a
+  // conversion reads a field off the alignment of its own type from an aligned
+  // copy.
   const size_t fsize = dtype == 0 ? sizeof(double) : sizeof(float);
   const bool aligned = reinterpret_cast<uintptr_t>(f) % fsize == 0, same = (dtype == 0) == f64;
-  if (!same || !aligned || (ld != N && !c->reg_path)) {
+  if (!same || !aligned) {
     if (!c->Fconv) CK(cudaMalloc(&c->Fconv, (size_t)ld * N * esize(c->prec)), "cudaMalloc(source conversion)");
     if (!same && !aligned) {
       CK(stage_acquire(c), "order after the last asynchronous read");

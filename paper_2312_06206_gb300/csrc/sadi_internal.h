@@ -37,7 +37,7 @@ struct RhsParams {
   int g;
   int first;
   const void* F;   // optional source field (T, N x N, row pitch ldF) or nullptr
-  int ldF;         // the state's pitch, or N for a caller's field (register paths)
+  int ldF;         // the state's pitch, or N for a caller's field
   double fsc;      // its time factor cos(omega t_n + phase) for this step
   double gc1, gc3, gcs;   // coefficients of g kind 3
 };

@@ -369,8 +369,8 @@ k_rows_remainder(const cx<T>* __restrict__ S, Geom g, const cx<T>* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// B^n at grid index idx (row element k, convolution read from the row vector
-// e).  Wave (Sec. 3): conv + tau^2 (g(u^n) + f^n), or at n = 0
+// B^n at element k of a grid row (arrays of pitch ld, the source of its own
+// pitch; convolution read from the row vector e).  Wave (Sec. 3): conv + tau^2 (g(u^n) + f^n), or at n = 0
 // tau phi2 + (conv + tau^2 (g + f))/2, conv = -kappa tau^2 L_h u^n.
 // Diffusion: tau (g(u~) + f) - d + conv, with conv = -kappa tau L_h u~ (the
 // plain form transforms u~ itself), or in the compensated form (Ch: the
@@ -380,21 +380,22 @@ k_rows_remainder(const cx<T>* __restrict__ S, Geom g, const cx<T>* __restrict__ 
 // DIFF: the equation of the launch (a template parameter of the row kernel,
 // so that the wave step's epilogue carries none of the diffusion step's code).
 template <typename T, bool DIFF>
-__device__ __forceinline__ T rhs_at(const RhsParams& rp, const cx<T>* e, int k, size_t idx, const T* u,
+__device__ __forceinline__ T rhs_at(const RhsParams& rp, const cx<T>* e, size_t row, int k, int ld, const T* u,
                                     const T* uaux, const T* phi2, float* Ch, float* Cl) {
+  const size_t idx = row * ld + k;
   if constexpr (!DIFF) {
     T conv = real_view<T>(e, k);
     if (Ch) conv = acc_remainder<T>(Ch, Cl, idx, conv);
     const T uu = u[idx];
     T gsrc = g_of<T>(rp, uu);
-    if (rp.F) gsrc += T(rp.fsc) * static_cast<const T*>(rp.F)[idx];
+    if (rp.F) gsrc += T(rp.fsc) * static_cast<const T*>(rp.F)[row * rp.ldF + k];
     const T gg = T(rp.tau2) * gsrc;
     return rp.first ? T(rp.tau) * phi2[idx] + T(0.5) * (conv + gg) : conv + gg;
   }
   const T cd = real_view<T>(e, k);
   const T conv = Ch ? acc_remainder<T>(Ch, Cl, idx, cd) : cd;
   const T uu = u[idx];
-  T fsrc = rp.F ? T(rp.fsc) * static_cast<const T*>(rp.F)[idx] : T(0);
+  T fsrc = rp.F ? T(rp.fsc) * static_cast<const T*>(rp.F)[row * rp.ldF + k] : T(0);
   const T d = rp.first ? T(0) : (Ch ? uaux[idx] : uu - uaux[idx]);
   const T ut = uu + T(0.5) * d;
   const T b = conv + T(rp.tau2) * (g_of<T>(rp, ut) + fsrc) - d;
@@ -439,12 +440,12 @@ k_rows_solve(const cx<T>* __restrict__ S, const T* __restrict__ u, const T* __re
           const size_t row = (size_t)(row0 + v);
           const cx<T>* e = buf + v * vs;
           if (k < N) {
-            const T b = rhs_at<T, DIFF>(rp, e, k, row * g.ld + k, u, uaux, phi2, Ch, Cl);
+            const T b = rhs_at<T, DIFF>(rp, e, row, k, g.ld, u, uaux, phi2, Ch, Cl);
             W[row * g.ld + k] = b;
             split_bf16(b, Bh + row * ldp + k, Bl + row * ldp + k);
           }
           if (k2 < N) {
-            const T b = rhs_at<T, DIFF>(rp, e, k2, row * g.ld + k2, u, uaux, phi2, Ch, Cl);
+            const T b = rhs_at<T, DIFF>(rp, e, row, k2, g.ld, u, uaux, phi2, Ch, Cl);
             W[row * g.ld + k2] = b;
             split_bf16(b, Bh + row * ldp + k2, Bl + row * ldp + k2);
           }
@@ -463,8 +464,8 @@ k_rows_solve(const cx<T>* __restrict__ S, const T* __restrict__ u, const T* __re
         if (v < nrows) {
           const int row = row0 + v;
           const cx<T>* e = buf + v * vs;
-          if (k < N) ra[it] = rhs_at<T, DIFF>(rp, e, k, (size_t)row * g.ld + k, u, uaux, phi2, Ch, Cl);
-          if (k2 < N) rb[it] = rhs_at<T, DIFF>(rp, e, k2, (size_t)row * g.ld + k2, u, uaux, phi2, Ch, Cl);
+          if (k < N) ra[it] = rhs_at<T, DIFF>(rp, e, row, k, g.ld, u, uaux, phi2, Ch, Cl);
+          if (k2 < N) rb[it] = rhs_at<T, DIFF>(rp, e, row, k2, g.ld, u, uaux, phi2, Ch, Cl);
         }
       }
     }
