@@ -263,11 +263,11 @@ sadi_status sadi_autotune(sadi_ctx** ctxs, int count, int g, int flags) {
       double ms = 0;
       if ((st = time_group(grp, 5, &ms)) != SADI_OK) return st;
       if (!reg_path_supported(logNp, prec)) {
-        // coordinate descent over the shared-memory engine's decomposition;
-        // the column convolution may also run as three passes (kConvThreePass)
+        // coordinate descent over the shared-memory engine's decomposition
+        // (the dense form has no y-sweep tile); the column convolution may
+        // also run as three passes (kConvThreePass)
         Tiles t = grp[0]->tiles32;
-        bool tiled = false;
-        const int nfields = 3;
+        const int nfields = prec == SADI_PREC_FP32 ? 3 : 2;
         const int opts[3][5] = {{1, 2, 4, 8, 0}, {kConvThreePass, 1, 2, 4, 8}, {1, 2, 4, 8, 0}};
         for (int f = 0; f < nfields; ++f) {
           for (int v : opts[f]) {
@@ -283,11 +283,10 @@ sadi_status sadi_autotune(sadi_ctx** ctxs, int count, int g, int flags) {
             if (m2 < ms) {
               ms = m2;
               t = tt;
-              tiled = true;
             }
           }
         }
-        if (tiled) cd.t = t;
+        cd.t = t;
         log += std::string(" ") + prec_name(prec) +
                fmt("(tiles %.0f/%.0f/%.0f) %.4f ms", t.rows, t.conv_cols, t.solve_cols, ms);
       } else {
