@@ -1,4 +1,4 @@
-// blkfft.cuh -- block-wide register FFT of length L = R1 R2 R3 (512 .. 8192).
+// blkfft.cuh -- block-wide register FFT of length L = R1 R2 R3 (256 .. 2048).
 //
 // T = R2 R3 threads own a vector; thread t holds the elements t + T q in
 // registers x[q], q < E = R1, before and after the transform (frequencies in
@@ -11,8 +11,8 @@
 //      exp(-2 pi i t' k2 / T); in place (a thread writes what it has read)
 //   3. R3-point DFTs over t' -> k3; frequency k = k1 + R1 (k2 + R2 k3)
 // so two shared-memory round trips and three barriers per transform, where a
-// radix-8 engine with the vector in shared memory takes five round trips (and
-// its index arithmetic) at L = 8192.  Half-warps (8-byte accesses) read and
+// radix-8 engine with the vector in shared memory takes four round trips (and
+// its index arithmetic) at L = 2048.  Half-warps (8-byte accesses) read and
 // write 16 consecutive elements in levels 1 and 2 and a stride of T + 1 (odd)
 // in level 3: no bank conflicts.
 #pragma once
@@ -88,14 +88,6 @@ struct Radix<10> {
 template <>
 struct Radix<11> {
   static constexpr int R1 = 16, R2 = 8, R3 = 16;
-};
-template <>
-struct Radix<12> {
-  static constexpr int R1 = 16, R2 = 16, R3 = 16;
-};
-template <>
-struct Radix<13> {
-  static constexpr int R1 = 32, R2 = 16, R3 = 16;
 };
 
 template <int LOGL>

@@ -4,11 +4,12 @@
 // A sweep on N points solves a bordered system of N' = 2^k unknowns and adds
 // G ybot to each vector (ybot: its r bottom entries).  For small r the sweep
 // kernels add it themselves, one column of G per bottom entry.  From
-// r > kBorderInline on every vector would read the whole of G (N = 1500:
-// 3.3 MB per row), so the sweep kernels store ybot (r x N) instead and this
-// kernel multiplies 64 x 64 tiles, each operand element read once per 64
-// outputs: bound by the FP32 multiply-adds (N = 1500, r = 548: 1.2 G per
-// sweep).  Below the line the extra launch costs more than it saves.
+// r > kBorderInline on every vector would read the whole of G (N = 700: 0.9 MB
+// per row), so the sweep kernels store ybot (r x N) instead and this kernel
+// multiplies 64 x 64 tiles, each operand element read once per 64 outputs: bound
+// by the FP32 multiply-adds (N = 700, r = 324: 0.16 G per sweep; the step 124
+// us, 1485 with G read per vector).  Below the line the extra launch costs more
+// than it saves.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -22,7 +23,6 @@ constexpr int kTile = 64, kK = 16, kThreads = 256;
 // MODE 0: the x sweep by columns, W[k][row] += sum_p G[p][k] ybot[p][row].
 // MODE 1: the y sweep, uhat[j][i] = U[j][i] + sum_p G[p][j] ybot[p][i], and the
 // compensated leapfrog of its element (step_blk.cuh).
-// MODE 2: the x sweep by rows, W[row][k] += sum_p ybot[p][row] G[p][k].
 template <int MODE>
 __global__ void __launch_bounds__(kThreads) k_border(const __grid_constant__ RegBatch B) {
   __shared__ __align__(16) float sp[2][kK][kTile], sq[2][kK][kTile];
@@ -32,9 +32,8 @@ __global__ void __launch_bounds__(kThreads) k_border(const __grid_constant__ Reg
   if (r <= kBorderInline || m0 >= N || n0 >= N) return;
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   pdl_entry();
-  const float* P = MODE == 2 ? I.YB : I.G;
-  const float* Q = MODE == 2 ? I.G : I.YB;
-  const int ldp = MODE == 2 ? I.ld : N, ldq = MODE == 2 ? N : I.ld;
+  const float *P = I.G, *Q = I.YB;
+  const int ldp = N, ldq = I.ld;
   float acc[4][4] = {};
   // thread -> element (p, column) of a K block: 4 of each operand
   float pv[4], qv[4];
@@ -83,7 +82,7 @@ __global__ void __launch_bounds__(kThreads) k_border(const __grid_constant__ Reg
       const int n = n0 + 4 * tx + j;
       if (n >= N) break;
       const size_t at = (size_t)m * I.ld + n;
-      if constexpr (MODE != 1) {
+      if constexpr (MODE == 0) {
         I.W[at] += acc[i][j];
       } else {
         const float uh = reinterpret_cast<const float*>(I.S)[at] + acc[i][j];

@@ -178,9 +178,10 @@ sadi_status alloc_state(sadi_ctx* c) {
   // (the register paths' slots hold lds >= N rows each)
   const size_t ses = (c->prec != SADI_PREC_FP64 && c->g.Np <= 4096) ? sizeof(double) : es;
   const size_t sbytes = (size_t)c->g.N * c->g.Np * 2 * ses;
-  size_t rbytes = c->prec != SADI_PREC_FP64 ? (size_t)slot_rows(c->g.N) * c->g.Np * sizeof(float2) : 0;
+  size_t rbytes = reg_path_supported(c->g.logNp, c->prec) ? (size_t)slot_rows(c->g.N) * c->g.Np * sizeof(float2) : 0;
   // behind the slots: the bottom entries of the bordered solves
-  if (c->prec == SADI_PREC_FP32 && c->g.r > kBorderInline) rbytes += (size_t)c->g.r * c->g.ld * sizeof(float);
+  if (rbytes && c->prec == SADI_PREC_FP32 && c->g.r > kBorderInline)
+    rbytes += (size_t)c->g.r * c->g.ld * sizeof(float);
   // the direct path's V and Wm (their order in dir_inst)
   const size_t dbytes = (3 * (size_t)c->g.N + 2) * c->g.ld * es;
   if (c->prec != SADI_PREC_FP32_DENSE && dir_mode(c->g, c->prec == SADI_PREC_FP64) && dbytes > rbytes)
@@ -196,8 +197,8 @@ sadi_status alloc_state(sadi_ctx* c) {
   }
   const sadi_status sd = setup_direct(c);
   if (sd != SADI_OK) return sd;
-  // FP32 forms whose explicit tiles select the three-pass column convolution:
-  // its buffers and tables (kept once allocated)
+  // FP32 forms whose tiles select the three-pass column convolution (the
+  // default at N' = 8192): its buffers and tables (kept once allocated)
   if (c->prec != SADI_PREC_FP64 && !c->reg_path && c->tiles32.conv_cols == kConvThreePass) {
     const sadi_status s3 = ensure_conv3(c);
     if (s3 != SADI_OK) return s3;
@@ -329,7 +330,7 @@ sadi_status create_impl(int eq, int N, double alpha, double kappa, double tau, c
       {(void**)&c->G32, sizeof(float) * ((size_t)N * g.r + 1)},
       {(void**)&c->stage, sizeof(double) * nn},
       {(void**)&c->rtw1, sizeof(float2) * (3 * Np + kTw2)},
-      {(void**)&c->rlreg, sizeof(float) * (reg_lreg_elems(g) + reg_lnat_elems(g))},
+      {(void**)&c->rlreg, sizeof(float) * (reg_lreg_elems(g) + reg_lnat_elems(g) + 1)},
       {(void**)&c->rlamc, sizeof(float2) * Np},
       {(void**)&c->rlams, sizeof(float2) * Np},
       {(void**)&c->wd, sizeof(WdState)},
@@ -499,9 +500,8 @@ sadi_status sadi_set_initial(sadi_ctx* c, const double* phi1, const double* phi2
          "starting remainder");
     } else {
       StepTables<float> tb{c->stw32, c->tw32, c->lpb32, c->lams32, c->lamc32, c->G32, c3_of(c)};
-      Tiles tl = default_tiles<float>(c->g.Np, c->g.N);
-      if (!c->c3.ZE) tl.conv_cols = 1;   // the three-pass buffers exist for explicit tiles only
-      CK(launch_remainder<float>(c->g, tb, tl, static_cast<const float*>(c->ubuf[0]), ld, c->S, c->Chi, c->Clo, st),
+      CK(launch_remainder<float>(c->g, tb, default_tiles<float>(c->g.Np, c->g.N),
+                                 static_cast<const float*>(c->ubuf[0]), ld, c->S, c->Chi, c->Clo, st),
          "starting remainder");
     }
   }

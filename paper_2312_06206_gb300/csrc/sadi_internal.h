@@ -145,9 +145,8 @@ bool tiles_valid(const Geom& g, const Tiles& t);
 template <typename T>
 cudaError_t step_setup_attributes();
 
-// FP32 register-FFT paths: a row per part of a warp up to N' = 1024
-// (step_reg.cuh), per block from 2048 on (step_blk.cuh).  One instance of a
-// batch:
+// FP32 register-FFT paths: a row per part of a warp (step_reg.cuh) or per warp
+// or block (step_blk.cuh; blk_path).  One instance of a batch:
 // natural-order tables and the in-place double-float state.
 struct RegInst {
   const float2* tw1;    // [N'] two-level FFT twiddles exp(-2 pi i t k1 / N') at [k1 * TT + t] (regfft.cuh)
@@ -157,8 +156,8 @@ struct RegInst {
   const float2* tw;     // [2N'] exp(-2 pi i k / 2N')
   const float2* lam_s;  // [N'] natural order, scaled as the bit-reversed tables
   const float2* lam_c;  // [N']
-  const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled (kRegMaxLog)
-  const float* lnat;    // [(N'+1) * (N'+1)] symbol by x- and y-frequency 0 .. N', scaled (kBlkMinLog)
+  const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled (kr_cols_conv)
+  const float* lnat;    // [(N'+1) * (N'+1)] symbol by x- and y-frequency 0 .. N', scaled (kb_cols_conv)
   const float* G;       // [r * N] border correction, column q at G + q N
   float* u_hi;          // state: u = u_hi + u_lo (double-float), u_d = u^n - u^{n-1}
   float* u_lo;
@@ -166,7 +165,7 @@ struct RegInst {
   const float* phi2;
   float2* S;            // spectrum scratch, slot-major: S[k * lds + row]
   int lds;              // rows per slot, N rounded up to 8 (64-byte runs of a cluster's rows stay aligned)
-  float* W;             // N x N sweep scratch (by columns between the GS sweeps from N' = 2048 on)
+  float* W;             // N x N sweep scratch (by columns between the GS sweeps of step_blk.cuh)
   float* YB;            // bottom entries of the sweeps' bordered solves, r x ld (r > kBorderInline)
   const float* F;       // optional source field (N x N, row pitch ldF) or nullptr
   int ldF;
@@ -191,17 +190,18 @@ constexpr int kMaxBatch = 32;
 // border ranks up to which the sweep kernels add the border correction
 // themselves (above: border.cuh, one more launch per sweep)
 constexpr int kBorderInline = 32;
-// passed by value as a __grid_constant__ kernel parameter (about 4 KB)
+// passed by value as a __grid_constant__ kernel parameter (about 8 KB)
 struct RegBatch {
   int count;
   RegInst in[kMaxBatch];
 };
 // FFT lengths of the two register paths: step_reg.cuh (a row per part of a warp)
-// up to 2^kRegMaxLog, step_blk.cuh (a row per warp or more) from 2^kBlkMinLog
-// (reg_path_supported: to 1024 in the GS form, 2048 in the dense form);
-// explicit tiles select the shared-memory engine from 2^kTilesMinLog on (the
-// dense form at 2048; the others run on it anyway).
-constexpr int kRegMaxLog = 10, kBlkMinLog = 8, kTilesMinLog = 11;
+// below 2^kBlkMinLog, and the dense form's row kernels at 2^kRegMaxLog;
+// step_blk.cuh (a row per warp or more) from 2^kBlkMinLog to 2^kBlkMaxLog
+// (reg_path_supported: to 1024 in the GS form, 2048 in the dense form).
+// Explicit tiles select the shared-memory engine from 2^kTilesMinLog on (the
+// dense form at 2048; longer transforms run on it anyway).
+constexpr int kRegMaxLog = 10, kBlkMinLog = 8, kBlkMaxLog = 11, kTilesMinLog = 11;
 // whether step_blk.cuh serves a context, else step_reg.cuh.  From N' = 256 on it
 // measured faster for one instance and for many (us per step, step_reg.cuh ->
 // step_blk.cuh: GS N = 255 1 / 16 instances 31 -> 21 / 63 -> 58, N = 511 68 ->
@@ -224,8 +224,10 @@ cudaError_t launch_step_reg(const RegBatch& b, int logNp, bool blk, int max_n, c
 // (N'), btw1h (N'), btw2 (kTw2); and in sym: lreg (reg_lreg_elems floats) and
 // lnat (reg_lnat_elems), each where its path exists
 constexpr int kTw2 = 256;
-inline size_t reg_lreg_elems(const Geom& g) { return g.logNp <= kRegMaxLog ? (size_t)(g.Np + 1) * 2 * g.Np : 0; }
-inline size_t reg_lnat_elems(const Geom& g) { return g.logNp >= kBlkMinLog ? (size_t)(g.Np + 1) * (g.Np + 1) : 0; }
+inline size_t reg_lreg_elems(const Geom& g) { return g.logNp < kBlkMinLog ? (size_t)(g.Np + 1) * 2 * g.Np : 0; }
+inline size_t reg_lnat_elems(const Geom& g) {
+  return g.logNp >= kBlkMinLog && g.logNp <= kBlkMaxLog ? (size_t)(g.Np + 1) * (g.Np + 1) : 0;
+}
 cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, const double2* lamc64,
                            const double2* lams64, float2* tw, float* sym, float2* lamc_nat, float2* lams_nat,
                            cudaStream_t st);

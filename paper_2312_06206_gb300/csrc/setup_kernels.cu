@@ -472,11 +472,10 @@ cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, cons
     case 9: blk(bf::BlkFFT<9>{}); break;
     case 10: blk(bf::BlkFFT<10>{}); break;
     case 11: blk(bf::BlkFFT<11>{}); break;
-    case 12: blk(bf::BlkFFT<12>{}); break;
-    case 13: blk(bf::BlkFFT<13>{}); break;
     default: break;
   }
   const size_t n = nreg > nfold ? nreg : nfold;
+  if (n == 0) return cudaSuccess;   // no register path at this length
   k_reg_tables<<<nblk(n, 256), 256, 0, st>>>(g, lnat, scale, 1 << (g.logNp / 2), T, R3, lamc64, lams64, tw, sym, nreg,
                                              sym + nreg, nfold, lamc_nat, lams_nat);
   return cudaGetLastError();

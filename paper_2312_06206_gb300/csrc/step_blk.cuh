@@ -18,15 +18,12 @@
 // of V rows, 64 or 32 bytes.  This replaces the two transpose passes of the shared-memory
 // engine's y sweep and its 8-byte column gathers.
 //
-// Measured against the shared-memory engine (us per launch, GB300): N = 4095
-// row FFT 145 -> 93, convolution 407 -> 157, B^n 258 -> 177, GS rows 537 ->
-// 370, y sweep 488 (with its transposes) -> 292; N = 8191 row FFT 681 -> 415,
-// convolution 1822 (three passes) -> 737, GS rows 2649 -> 1750, y sweep 2241
-// -> 1260; N = 2047, four instances: 80 + 192 + 264 -> 75 + 175 + 170 against
-// the 64-elements-per-lane kernels this replaces there.  Instructions per
-// element and transform fell from 134 to about 50; what bounds the kernels now
-// is the latency of the table loads and barriers at 16 to 32 warps per SM
-// (issue 50%, L1 55%, FP32 pipe 38% in the convolution).
+// Measured (GB300): N = 2047 dense, four instances, row FFT, convolution and
+// B^n 80 + 192 + 264 -> 75 + 175 + 170 us against the 64-elements-per-lane
+// kernels this replaces there; steps of the other lengths at blk_path.  Longer
+// transforms keep the shared-memory engine (reg_path_supported).  What bounds
+// the kernels is the latency of the table loads and barriers at 16 to 32 warps
+// per SM.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -114,22 +111,25 @@ struct Cfg {
   static_assert(V * P1 <= 2 * ELEMS, "the float exchange buffer fits too");
   static constexpr size_t bytes = (size_t)R * ELEMS * sizeof(float2);
   static constexpr size_t bytes_conv = (size_t)(F::BUF + (LOGL <= 10 ? F::BUF : F::L)) * sizeof(float2);
-  // resident blocks promised to the compiler (its register budget), measured
-  // at N = 4095 (us per launch at 2 / 3 / 4 blocks of 256 threads): r2c 109 /
-  // 100 / 94, dense B^n 208 / 179 / 177, GS rows 378 / 362 / -, columns 289 /
-  // 312.  E = 32 (N' = 8192) needs 128 registers.  Seven N = 511 instances,
-  // dense B^n: 18 us at 64 registers, 21 at 85.
+  // resident blocks promised to the compiler (its register budget): 64
+  // registers a thread for the row FFT and, at N' = 512 and 2048, the dense
+  // B^n kernel (seven N = 511 instances: 18 us, 21 at 85 registers), 128 for
+  // the sweeps
   static constexpr int kM = 256 / F::T;   // rows for each 256 threads
   static constexpr int per(int rows) { return rows / R > 0 ? rows / R : 1; }
-  static constexpr int kR2cBlocks = per(LOGL == 13 ? 2 : 4 * kM);
-  static constexpr int kDenseBlocks = per(LOGL == 13 ? 2 : LOGL >= 11 ? 4 * kM : LOGL == 9 ? 4 * kM : 2 * kM);
-  static constexpr int kGsBlocks = per(LOGL == 13 ? 2 : LOGL >= 11 ? 3 * kM : 2 * kM);
+  static constexpr int kR2cBlocks = per(4 * kM);
+  static constexpr int kDenseBlocks = per(LOGL == 11 || LOGL == 9 ? 4 * kM : 2 * kM);
+  static constexpr int kGsBlocks = per(2 * kM);
   static constexpr int kColsBlocks = per(2 * kM);
   // the two convolution kernels: both halves in one block up to N' = 1024
   // (29 us at 4 blocks a SM, 30 at 5, 31 at 6 for three N = 1023 instances),
   // one after the other above
   static constexpr bool kConvSplit = LOGL <= 10;
-  static constexpr int kConvBlocks = LOGL == 10 ? 4 : LOGL == 9 ? 6 : LOGL == 8 ? 12 : LOGL == 13 ? 1 : 2 * kM;
+  // what runs at this length (launch_step_reg): the dense form's row kernels, the
+  // GS sweeps, and border ranks above kBorderInline among them (below N' = 1024
+  // those take dense sweeps, dir_mode)
+  static constexpr bool kDense = LOGL != 10, kGS = LOGL <= 10, kBorder = LOGL == 10;
+  static constexpr int kConvBlocks = LOGL == 10 ? 4 : LOGL == 9 ? 6 : LOGL == 8 ? 12 : 2 * kM;
 };
 
 // Exchange between the V rows of a cluster: the barrier over all of them
@@ -288,13 +288,11 @@ kb_cols_conv(const __grid_constant__ RegBatch B) {
   });
 }
 
-// The same with one half after the other on T threads, from N' = 2048 on: the
-// even half's result waits in shared memory (each thread its own elements),
-// and the odd half reads the column again (from L2).  Independent blocks with
-// their full registers overlap loads, transforms and stores, where the split
-// kernel's one block of 512 threads an SM ran in lockstep (N = 4095 193 -> 157
-// us, N = 8191, 255 registers and no spills, 1098 -> 737); more blocks than two
-// an SM take L1 from the tables and lose (174 at three, 205 at four).
+// The same with one half after the other on T threads, at N' = 2048: the even
+// half's result waits in shared memory (each thread its own elements), and the
+// odd half reads the column again (from L2).  Independent blocks with their full
+// registers overlap loads, transforms and stores (N = 2047 39 -> 37 us); below,
+// the split kernel's smaller blocks do that too (N = 1023 15.9 us, 16.3 so).
 template <int LOGL>
 __global__ void __launch_bounds__(BlkFFT<LOGL>::T, Cfg<LOGL>::kConvBlocks)
 kb_cols_conv_seq(const __grid_constant__ RegBatch B) {
@@ -376,10 +374,12 @@ __device__ __forceinline__ void gs_solve(float2* x, float* y, float2* sm, int t,
     y[q] = x[q].x + sm[F::L - 1 - (t + F::T * q)].y;
   });
   const int N = I.N, r = I.r;
-  if (r > kBorderInline) {
-    if (vec < N)
-      for (int p = t; p < r; p += F::T) I.YB[(size_t)p * I.ld + vec] = sm[N + p].x + sm[r - 1 - p].y;
-    return;
+  if constexpr (Cfg<LOGL>::kBorder) {
+    if (r > kBorderInline) {
+      if (vec < N)
+        for (int p = t; p < r; p += F::T) I.YB[(size_t)p * I.ld + vec] = sm[N + p].x + sm[r - 1 - p].y;
+      return;
+    }
   }
 #pragma unroll 1
   for (int p = 0; p < r; ++p) {
@@ -624,15 +624,17 @@ kb_cols_solve(const __grid_constant__ RegBatch B) {
   const int vv = t % C::V, s0 = t / C::V;
   if (i0 + vv >= N) return;
   const float* src = smf + vv * C::P1 + s0;
-  if (I.r > kBorderInline) {
-    // uhat short of its border correction, by rows, for border.cuh
-    float* U = reinterpret_cast<float*>(I.S);
+  if constexpr (C::kBorder) {
+    if (I.r > kBorderInline) {
+      // uhat short of its border correction, by rows, for border.cuh
+      float* U = reinterpret_cast<float*>(I.S);
 #pragma unroll 4
-    for (int e = 0; e < F::E; ++e) {
-      const int j = rank * C::SEG + s0 + F::T / C::V * e;
-      if (j < N) U[(size_t)j * I.ld + i0 + vv] = src[F::T / C::V * e];
+      for (int e = 0; e < F::E; ++e) {
+        const int j = rank * C::SEG + s0 + F::T / C::V * e;
+        if (j < N) U[(size_t)j * I.ld + i0 + vv] = src[F::T / C::V * e];
+      }
+      return;
     }
-    return;
   }
   const int first = I.first;
 #pragma unroll 1
@@ -691,14 +693,17 @@ cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
   static LaunchCache attr_done[kLauncherDevices];
   const int dev = device_slot();
   if (dev < 0) return cudaErrorInvalidDevice;
+  if (dense ? !C::kDense : !C::kGS) return cudaErrorInvalidValue;
   cudaError_t e;
   if (!attr_done[dev].load(std::memory_order_acquire)) {
     auto room = [](auto kernel, size_t bytes) {
       return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    if ((e = room(kb_rows_r2c<LOGL>, C::bytes)) || (e = room(kb_rows_solve<LOGL, false>, C::bytes)) || (e = room(kb_rows_solve<LOGL, true>, C::bytes)) ||
-        (e = room(kb_cols_solve<LOGL>, C::bytes)))
-      return e;
+    if ((e = room(kb_rows_r2c<LOGL>, C::bytes))) return e;
+    if constexpr (C::kDense)
+      if ((e = room(kb_rows_solve<LOGL, true>, C::bytes))) return e;
+    if constexpr (C::kGS)
+      if ((e = room(kb_rows_solve<LOGL, false>, C::bytes)) || (e = room(kb_cols_solve<LOGL>, C::bytes))) return e;
     attr_done[dev].store(1, std::memory_order_release);
   }
   // every kernel of the step is a programmatic dependent of the one before
@@ -726,14 +731,20 @@ cudaError_t launch_blk_impl(const RegBatch& b, int max_n, cudaStream_t st, cudaE
   if (ev) cudaEventRecord(ev[1], st);
   if ((e = launch_blk_conv<LOGL>(b, st))) return e;
   if (ev) cudaEventRecord(ev[2], st);
-  if (dense) return launch(kb_rows_solve<LOGL, true>, rgrid, C::R * F::T, C::bytes);
-  const bool border = border::any(b);
-  if ((e = launch(kb_rows_solve<LOGL, false>, rgrid, C::R * F::T, C::bytes))) return e;
-  if (border && (e = border::launch<0>(b, max_n, st))) return e;
-  if (ev) cudaEventRecord(ev[3], st);
-  if ((e = launch(kb_cols_solve<LOGL>, rgrid, C::R * F::T, C::bytes))) return e;
-  if (border && (e = border::launch<1>(b, max_n, st))) return e;
-  if (ev) cudaEventRecord(ev[4], st);
+  if constexpr (C::kDense)
+    if (dense) return launch(kb_rows_solve<LOGL, true>, rgrid, C::R * F::T, C::bytes);
+  if constexpr (C::kGS) {
+    const bool border = border::any(b);
+    if (border && !C::kBorder) return cudaErrorInvalidValue;
+    if ((e = launch(kb_rows_solve<LOGL, false>, rgrid, C::R * F::T, C::bytes))) return e;
+    if constexpr (C::kBorder)
+      if (border && (e = border::launch<0>(b, max_n, st))) return e;
+    if (ev) cudaEventRecord(ev[3], st);
+    if ((e = launch(kb_cols_solve<LOGL>, rgrid, C::R * F::T, C::bytes))) return e;
+    if constexpr (C::kBorder)
+      if (border && (e = border::launch<1>(b, max_n, st))) return e;
+    if (ev) cudaEventRecord(ev[4], st);
+  }
   return cudaSuccess;
 }
 
