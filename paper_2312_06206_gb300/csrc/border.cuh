@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kThreads) k_border(const __grid_constant__ Reg
   if (r <= kBorderInline || m0 >= N || n0 >= N) return;
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   pdl_entry();
-  const float *P = I.G, *Q = I.YB;
+  const float *P = I.G, *Q = ybot_of(I, N + r);   // N' = N + r
   const int ldp = N, ldq = I.ld;
   float acc[4][4] = {};
   // thread -> element (p, column) of a K block: 4 of each operand

@@ -50,7 +50,7 @@ T* dalloc(size_t n, cudaError_t* e) {
 }
 
 void free_all(sadi_ctx* c) {
-  void* ptrs[] = {c->rtw1, c->rlreg, c->rlamc, c->rlams, c->stw64, c->stw32, c->a1,     c->a2d,    c->cgen,   c->lnat,   c->tw64,   c->tw32, c->lpb64,
+  void* ptrs[] = {c->rtw1, c->rsym, c->rlamc, c->rlams, c->stw64, c->stw32, c->a1,     c->a2d,    c->cgen,   c->lnat,   c->tw64,   c->tw32, c->lpb64,
                   c->lpb32,  c->lamc64, c->lams64, c->lamc32, c->lams32, c->G64,  c->G32,
                   c->ubuf[0], c->ubuf[1], c->ulo, c->F, c->phi2, c->S,      c->W,      c->stage};
   for (void* p : ptrs)
@@ -330,7 +330,7 @@ sadi_status create_impl(int eq, int N, double alpha, double kappa, double tau, c
       {(void**)&c->G32, sizeof(float) * ((size_t)N * g.r + 1)},
       {(void**)&c->stage, sizeof(double) * nn},
       {(void**)&c->rtw1, sizeof(float2) * (3 * Np + kTw2)},
-      {(void**)&c->rlreg, sizeof(float) * (reg_lreg_elems(g) + reg_lnat_elems(g) + 1)},
+      {(void**)&c->rsym, sizeof(float) * (reg_lreg_elems(g) + reg_lnat_elems(g) + 1)},
       {(void**)&c->rlamc, sizeof(float2) * Np},
       {(void**)&c->rlams, sizeof(float2) * Np},
       {(void**)&c->wd, sizeof(WdState)},
@@ -361,7 +361,7 @@ sadi_status create_impl(int eq, int N, double alpha, double kappa, double tau, c
     return bail(SADI_ENOTSPD);
   }
   c->reg_path = wants_reg_path(c);
-  if ((e = run_reg_tables(g, c->lnat, scale, c->lamc64, c->lams64, c->rtw1, c->rlreg, c->rlamc, c->rlams, st)))
+  if ((e = run_reg_tables(g, c->lnat, scale, c->lamc64, c->lams64, c->rtw1, c->rsym, c->rlamc, c->rlams, st)))
     return bail(cuda_fail(c, e, "register-path tables"));
   if ((e = step_setup_attributes<float>())) return bail(cuda_fail(c, e, "kernel attributes"));
   if ((e = step_setup_attributes<double>())) return bail(cuda_fail(c, e, "kernel attributes"));
@@ -569,16 +569,11 @@ RhsParams rhs_of(const sadi_ctx* c, long long n) {
 
 RegInst reg_inst(const sadi_ctx* c) {
   RegInst r{};
-  const int Np = c->g.Np;
   r.tw1 = c->rtw1;
-  r.btw1 = r.tw1 + Np;
-  r.btw1h = r.btw1 + Np;
-  r.btw2 = r.btw1h + Np;
   r.tw = c->tw32;
   r.lam_s = c->rlams;
   r.lam_c = c->rlamc;
-  r.lreg = c->rlreg;
-  r.lnat = c->rlreg + reg_lreg_elems(c->g);
+  r.sym = c->rsym;
   r.G = c->G32;
   r.u_hi = static_cast<float*>(c->ubuf[0]);
   r.u_d = static_cast<float*>(c->ubuf[1]);
@@ -587,7 +582,6 @@ RegInst reg_inst(const sadi_ctx* c) {
   r.S = static_cast<float2*>(c->S);
   const bool blk = blk_path(c->g.logNp, c->prec == SADI_PREC_FP32_DENSE);
   r.lds = blk ? slot_rows(c->g.N) : c->g.N;
-  r.YB = reinterpret_cast<float*>(r.S + (size_t)slot_rows(c->g.N) * c->g.Np);
   r.W = static_cast<float*>(c->W);
   r.N = c->g.N;
   r.ld = c->g.ld;

@@ -43,7 +43,7 @@ struct sadi_ctx {
   bool tiles_explicit = false;
   // FP32 register-FFT path tables
   float2* rtw1 = nullptr;
-  float* rlreg = nullptr;
+  float* rsym = nullptr;
   float2* rlamc = nullptr;
   float2* rlams = nullptr;
   bool reg_path = false;

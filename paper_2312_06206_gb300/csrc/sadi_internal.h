@@ -147,33 +147,36 @@ cudaError_t step_setup_attributes();
 
 // FP32 register-FFT paths: a row per part of a warp (step_reg.cuh) or per warp
 // or block (step_blk.cuh; blk_path).  One instance of a batch:
-// natural-order tables and the in-place double-float state.
+// natural-order tables and the in-place double-float state.  Behind the
+// spectrum's N' slots of lds rows lie, for r > kBorderInline, the bottom entries
+// of the sweeps' bordered solves, r x ld floats (ybot_of).
 struct RegInst {
-  const float2* tw1;    // [N'] two-level FFT twiddles exp(-2 pi i t k1 / N') at [k1 * TT + t] (regfft.cuh)
-  // tables of blkfft.cuh: [N'] exp(-2 pi i t k1 / N') at [k1 * T + t], the same
-  // at half frequencies (k1 + 1/2), and the second level's at [k2 * R3 + t']
-  const float2 *btw1, *btw1h, *btw2;
+  // [N'] two-level FFT twiddles exp(-2 pi i t k1 / N') at [k1 * TT + t]
+  // (regfft.cuh), and behind them the tables of blkfft.cuh: [N'] exp(-2 pi i t
+  // k1 / N') at [k1 * T + t], [N'] the same at half frequencies (k1 + 1/2), and
+  // the second level's at [k2 * R3 + t'] (btw1, btw1h, btw2 in step_blk.cuh)
+  const float2* tw1;
   const float2* tw;     // [2N'] exp(-2 pi i k / 2N')
   const float2* lam_s;  // [N'] natural order, scaled as the bit-reversed tables
   const float2* lam_c;  // [N']
-  const float* lreg;    // [(N'+1) * 2 * N'] symbol rows by x-frequency, even/odd halves, scaled (kr_cols_conv)
-  const float* lnat;    // [(N'+1) * (N'+1)] symbol by x- and y-frequency 0 .. N', scaled (kb_cols_conv)
+  // symbol, scaled: [(N'+1) * 2 * N'] rows by x-frequency, even/odd halves
+  // (kr_cols_conv, reg_lreg_elems), or [(N'+1) * (N'+1)] by x- and y-frequency
+  // 0 .. N' (kb_cols_conv, reg_lnat_elems)
+  const float* sym;
   const float* G;       // [r * N] border correction, column q at G + q N
   float* u_hi;          // state: u = u_hi + u_lo (double-float), u_d = u^n - u^{n-1}
   float* u_lo;
   float* u_d;
   const float* phi2;
   float2* S;            // spectrum scratch, slot-major: S[k * lds + row]
-  int lds;              // rows per slot, N rounded up to 8 (64-byte runs of a cluster's rows stay aligned)
   float* W;             // N x N sweep scratch (by columns between the GS sweeps of step_blk.cuh)
-  float* YB;            // bottom entries of the sweeps' bordered solves, r x ld (r > kBorderInline)
   const float* F;       // optional source field (N x N, row pitch ldF) or nullptr
-  int ldF;
   float* C_hi;          // incremental remainder -kappa tau^2 L_h u^n (double-float)
   float* C_lo;
   unsigned short* Bh;   // dense-inverse form: BF16 split of B^n (ld ldp, zero-padded)
   unsigned short* Bl;
   int ldp;
+  int lds;              // rows per slot; step_blk.cuh: N rounded up to 8 (64-byte runs of a cluster's rows stay aligned)
   // dense form: the sweep GEMM's panel and tile counters (ndep ints), zeroed
   // by the B^n kernel for the GEMM launched after it (nullptr: none)
   int* dep;
@@ -183,14 +186,20 @@ struct RegInst {
   float tau, tau2;
   float fsc;            // time factor of the source for this step
   int gkind, first;
+  int ldF;
   float gc1, gc3, gcs;  // coefficients of g kind 3 (gc1 u + gc3 u^3 + gcs sin u)
   int eq;               // 0 wave, 1 diffusion (RhsParams::eq); tau2 = tau^2 or tau
 };
+#ifdef __CUDACC__
+__device__ __forceinline__ float* ybot_of(const RegInst& I, int Np) {
+  return reinterpret_cast<float*>(I.S + (size_t)I.lds * Np);
+}
+#endif
 constexpr int kMaxBatch = 32;
 // border ranks up to which the sweep kernels add the border correction
 // themselves (above: border.cuh, one more launch per sweep)
 constexpr int kBorderInline = 32;
-// passed by value as a __grid_constant__ kernel parameter (about 8 KB)
+// passed by value as a __grid_constant__ kernel parameter (6.6 KB)
 struct RegBatch {
   int count;
   RegInst in[kMaxBatch];
@@ -221,8 +230,8 @@ cudaError_t launch_step_reg(const RegBatch& b, int logNp, bool blk, int max_n, c
                             bool dense = false);
 // natural-order FP32 tables of the register paths from the FP64 setup
 // products, behind one another in tw: tw1 (N' entries, step_reg.cuh), btw1
-// (N'), btw1h (N'), btw2 (kTw2); and in sym: lreg (reg_lreg_elems floats) and
-// lnat (reg_lnat_elems), each where its path exists
+// (N'), btw1h (N'), btw2 (kTw2); and in sym the one of the two symbols that the
+// column convolution of this length reads (RegInst::sym)
 constexpr int kTw2 = 256;
 inline size_t reg_lreg_elems(const Geom& g) { return g.logNp < kBlkMinLog ? (size_t)(g.Np + 1) * 2 * g.Np : 0; }
 inline size_t reg_lnat_elems(const Geom& g) {

@@ -364,12 +364,12 @@ __global__ void k_border_G(const double* __restrict__ X, const double* __restric
   G32[at] = (float)(-acc);
 }
 
-// Register-path tables (layout: run_reg_tables).  TT, T: threads per vector of
+// Register-path tables (layout: run_reg_tables; one of the two symbols).  TT, T: threads per vector of
 // regfft.cuh and blkfft.cuh (T = 0: no block path at this length).
 // lam*_nat[k] = lam*[brev(k)].
 __global__ void k_reg_tables(Geom g, const double* __restrict__ lnat, double scale, int TT, int T, int R3,
                              const double2* __restrict__ lamc64, const double2* __restrict__ lams64, float2* tw,
-                             float* lreg, size_t nreg, float* lfold, size_t nfold, float2* lamc_nat, float2* lams_nat) {
+                             float* lreg, size_t nreg, float* symnat, size_t nfold, float2* lamc_nat, float2* lams_nat) {
   const int Np = g.Np, logNp = g.logNp, P = g.P;
   const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   auto root = [](double num, double den) {   // exp(-2 pi i num / den)
@@ -390,7 +390,7 @@ __global__ void k_reg_tables(Geom g, const double* __restrict__ lnat, double sca
     lamc_nat[k] = make_float2((float)a.x, (float)a.y);
     lams_nat[k] = make_float2((float)b.x, (float)b.y);
   }
-  if (idx < nfold) lfold[idx] = (float)(scale * lnat[idx]);
+  if (idx < nfold) symnat[idx] = (float)(scale * lnat[idx]);
   if (idx < nreg) {
     const int m = (int)(idx % Np);
     const int h = (int)((idx / Np) % 2);
@@ -477,7 +477,7 @@ cudaError_t run_reg_tables(const Geom& g, const double* lnat, double scale, cons
   const size_t n = nreg > nfold ? nreg : nfold;
   if (n == 0) return cudaSuccess;   // no register path at this length
   k_reg_tables<<<nblk(n, 256), 256, 0, st>>>(g, lnat, scale, 1 << (g.logNp / 2), T, R3, lamc64, lams64, tw, sym, nreg,
-                                             sym + nreg, nfold, lamc_nat, lams_nat);
+                                             sym, nfold, lamc_nat, lams_nat);
   return cudaGetLastError();
 }
 

@@ -83,6 +83,14 @@ __device__ __forceinline__ void st_peer(unsigned a, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 
+// Tables of blkfft.cuh (RegInst::tw1).
+template <int LOGL>
+__device__ __forceinline__ const float2* btw1(const RegInst& I) { return I.tw1 + BlkFFT<LOGL>::L; }
+template <int LOGL>
+__device__ __forceinline__ const float2* btw1h(const RegInst& I) { return I.tw1 + 2 * BlkFFT<LOGL>::L; }
+template <int LOGL>
+__device__ __forceinline__ const float2* btw2(const RegInst& I) { return I.tw1 + 3 * BlkFFT<LOGL>::L; }
+
 // Barrier of the T threads of a row (rl: the row's place in its block).
 template <int T>
 __device__ __forceinline__ void row_sync(int rl) {
@@ -193,7 +201,7 @@ kb_rows_r2c(const __grid_constant__ RegBatch B) {
     }
     x[q] = v;
   });
-  F::fwd(x, sm, t, I.btw1, false, I.btw2, sync);
+  F::fwd(x, sm, t, btw1<LOGL>(I), false, btw2<LOGL>(I), sync);
   static_for<0, F::E>([&](auto qc) { sm[t + F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
   sync();
   // X[k] = (Z[k] + conj Z[-k]) / 2 + w^k (Z[k] - conj Z[-k]) / (2 i); slot 0 = X[0] + i X[N']
@@ -257,16 +265,16 @@ kb_cols_conv(const __grid_constant__ RegBatch B) {
     });
   }
   // odd half: frequencies m + 1/2 of the length-L transform
-  const float2* tw1 = h ? I.btw1h : I.btw1;
-  F::fwd(x, sm, t, tw1, h, I.btw2, sync);
+  const float2* tw1 = h ? btw1h<LOGL>(I) : btw1<LOGL>(I);
+  F::fwd(x, sm, t, tw1, h, btw2<LOGL>(I), sync);
   // the symbol at y frequency 2 m + h, stored for 0 .. N' (it is even)
-  const float* lam = I.lnat + (size_t)kx * (F::L + 1);
+  const float* lam = I.sym + (size_t)kx * (F::L + 1);
   static_for<0, F::E>([&](auto qc) {
     constexpr int q = decltype(qc)::value;
     const int k2 = 2 * (t + F::T * q) + h;
     x[q] = cscale(x[q], __ldg(&lam[q < F::E / 2 ? k2 : 2 * F::L - k2]));
   });
-  F::inv(x, sm, t, tw1, h, I.btw2, sync);
+  F::inv(x, sm, t, tw1, h, btw2<LOGL>(I), sync);
   // even + odd half: the odd threads hand over the rows of
   // q < E/2, the even threads the others, and each finishes its own rows
   constexpr int HE = F::E / 2;
@@ -322,15 +330,15 @@ kb_cols_conv_seq(const __grid_constant__ RegBatch B) {
         x[q] = j < N ? col[j] : make_float2(0.f, 0.f);
       });
     }
-    const float2* tw1 = h ? I.btw1h : I.btw1;
-    F::fwd(x, sm, t, tw1, h, I.btw2, sync);
-    const float* lam = I.lnat + (size_t)kx * (F::L + 1);
+    const float2* tw1 = h ? btw1h<LOGL>(I) : btw1<LOGL>(I);
+    F::fwd(x, sm, t, tw1, h, btw2<LOGL>(I), sync);
+    const float* lam = I.sym + (size_t)kx * (F::L + 1);
     static_for<0, F::E>([&](auto qc) {
       constexpr int q = decltype(qc)::value;
       const int k2 = 2 * (t + F::T * q) + h;
       x[q] = cscale(x[q], __ldg(&lam[q < F::E / 2 ? k2 : 2 * F::L - k2]));
     });
-    F::inv(x, sm, t, tw1, h, I.btw2, sync);
+    F::inv(x, sm, t, tw1, h, btw2<LOGL>(I), sync);
     if (h == 0) static_for<0, F::E>([&](auto qc) { keep[F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
   }
   static_for<0, F::E>([&](auto qc) {
@@ -350,7 +358,7 @@ kb_cols_conv_seq(const __grid_constant__ RegBatch B) {
 // factors Q and Q^H are the half-frequency shift of the first pair), then
 // y[q] = (H^-1 v)[k], k = t + T q: Re vhat[k] + Im vhat[N'-1-k] + the border
 // correction sum_p G[k, p] ybot[p], ybot[p] = Re vhat[N+p] + Im vhat[r-1-p];
-// for r > kBorderInline ybot of vector vec goes to YB, for border.cuh.
+// for r > kBorderInline ybot of vector vec is stored for border.cuh.
 template <int LOGL, typename Sync>
 __device__ __forceinline__ void gs_solve(float2* x, float* y, float2* sm, int t, int vec, const RegInst& I, Sync sync) {
   using F = BlkFFT<LOGL>;
@@ -359,13 +367,13 @@ __device__ __forceinline__ void gs_solve(float2* x, float* y, float2* sm, int t,
 #pragma unroll 1
   for (int round = 0; round < 2; ++round) {
     const float2* lam = round == 0 ? I.lam_s : I.lam_c;
-    const float2* tw1 = round == 0 ? I.btw1h : I.btw1;
-    F::fwd(x, sm, t, tw1, round == 0, I.btw2, sync);
+    const float2* tw1 = round == 0 ? btw1h<LOGL>(I) : btw1<LOGL>(I);
+    F::fwd(x, sm, t, tw1, round == 0, btw2<LOGL>(I), sync);
     static_for<0, F::E>([&](auto qc) {
       constexpr int q = decltype(qc)::value;
       x[q] = cmul(x[q], __ldg(&lam[t + F::T * q]));
     });
-    F::inv(x, sm, t, tw1, round == 0, I.btw2, sync);
+    F::inv(x, sm, t, tw1, round == 0, btw2<LOGL>(I), sync);
   }
   static_for<0, F::E>([&](auto qc) { sm[t + F::T * decltype(qc)::value] = x[decltype(qc)::value]; });
   sync();
@@ -376,8 +384,9 @@ __device__ __forceinline__ void gs_solve(float2* x, float* y, float2* sm, int t,
   const int N = I.N, r = I.r;
   if constexpr (Cfg<LOGL>::kBorder) {
     if (r > kBorderInline) {
+      float* yb = ybot_of(I, F::L);
       if (vec < N)
-        for (int p = t; p < r; p += F::T) I.YB[(size_t)p * I.ld + vec] = sm[N + p].x + sm[r - 1 - p].y;
+        for (int p = t; p < r; p += F::T) yb[(size_t)p * I.ld + vec] = sm[N + p].x + sm[r - 1 - p].y;
       return;
     }
   }
@@ -458,7 +467,7 @@ kb_rows_solve(const __grid_constant__ RegBatch B) {
     x[q] = (q == 0 && t == 0) ? make_float2(0.5f * (Xk.x + Xk.y), 0.5f * (Xk.x - Xk.y)) : cadd(Ev, cmul_pi(Ov));
   });
   sync();
-  F::inv(x, sm, t, I.btw1, false, I.btw2, sync);
+  F::inv(x, sm, t, btw1<LOGL>(I), false, btw2<LOGL>(I), sync);
   // x[q], q < E/2, now holds the convolution at 2n, 2n + 1, n = t + T q.
   // Wave step: B = C + tau^2 (g(u) + f), n = 0: tau phi2 + (C + tau^2 (g + f))/2,
   // with C <- C + conv; diffusion: B = C + conv/2 + tau (g(u~) + f) - d,

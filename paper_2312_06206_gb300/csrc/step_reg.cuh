@@ -215,27 +215,25 @@ __device__ __forceinline__ float real_at(const float2* sm, int k) {
   return reinterpret_cast<const float*>(sm + pad32(k >> 1))[k & 1];
 }
 
-// The solve of one vector from vhat in shared memory (natural order):
-// y[q] = (H^-1 v)[k], k = t + TT q < N: Re vhat[k] + Im vhat[N'-1-k] plus the
-// border correction sum_p G[k, p] ybot[p], ybot[p] = Re vhat[N+p] +
-// Im vhat[r-1-p].  ybot is formed once per vector, in the real part of
-// vhat[N + p] (which nothing else reads), then each lane adds column p of G
-// to all its outputs: its loads of one p are independent and coalesced (rows
-// of G and ybot anew for every k before: at N = 399, r = 113 this took the step
-// from 313 to 163 us).  sync: the barrier of the vector's
-// threads.
+// The border correction of one vector (r > 0) from vhat in shared memory
+// (natural order): the real part of vhat[k] becomes y[k] = (H^-1 v)[k], k < N,
+// Re vhat[k] + Im vhat[N'-1-k] + sum_p G[k, p] ybot[p].  The same sum without the
+// last term at k = N + p is ybot[p].  Each lane adds column p of G to all its
+// outputs: its loads of one p are independent and coalesced (rows of G and ybot
+// anew for every k before: N = 95 54 -> 21 us per step, N = 127 32 -> 25).  sync:
+// the barrier of the vector's threads.
 template <int LOGL, typename Sync>
-__device__ __forceinline__ void gs_out_reg(float* y, float2* sm, int t, const RegInst& I, Sync sync) {
+__device__ __forceinline__ void gs_border_reg(float2* sm, int t, const RegInst& I, Sync sync) {
   using F = rf::RegFFT<float, LOGL>;
   const int N = I.N, r = I.r;
-  static_for<0, F::E>([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
+#pragma unroll 2
+  for (int q = 0; q < F::E; ++q) {
     const int k = t + F::TT * q;
-    y[q] = k < N ? sm[pad32(k)].x + sm[pad32(F::L - 1 - k)].y : 0.f;
-  });
-  if (r == 0) return;
-  for (int p = t; p < r; p += F::TT) sm[pad32(N + p)].x += sm[pad32(r - 1 - p)].y;
+    sm[pad32(k)].x += sm[pad32(F::L - 1 - k)].y;
+  }
   sync();
+  float y[F::E];
+  static_for<0, F::E>([&](auto qc) { y[decltype(qc)::value] = sm[pad32(t + F::TT * decltype(qc)::value)].x; });
 #pragma unroll 1
   for (int p = 0; p < r; ++p) {
     const float yb = sm[pad32(N + p)].x;
@@ -246,6 +244,17 @@ __device__ __forceinline__ void gs_out_reg(float* y, float2* sm, int t, const Re
       if (k < N) y[q] += __ldg(Gp + k) * yb;
     });
   }
+  static_for<0, F::E>([&](auto qc) {
+    constexpr int q = decltype(qc)::value;
+    const int k = t + F::TT * q;
+    if (k < N) sm[pad32(k)].x = y[q];
+  });
+}
+// (H^-1 v)[k] after it, or straight from vhat (r = 0)
+template <int LOGL>
+__device__ __forceinline__ float gs_out_reg(const float2* sm, int k, int r) {
+  const float y = sm[pad32(k)].x;
+  return r > 0 ? y : y + sm[pad32((1 << LOGL) - 1 - k)].y;
 }
 
 // ---------------------------------------------------------------------------
@@ -257,6 +266,7 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   using C = RowCfg<LOGL, BLOCK>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const RegInst& I = B.in[blockIdx.y];
+  const int lds = I.lds;   // once: a copy loop would read the parameter again for each element
   const int N = I.N;
   if ((int)blockIdx.x * C::VB >= N) return;
   const int v = threadIdx.x / F::TT, t = threadIdx.x % F::TT;
@@ -307,12 +317,12 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
     const float2 Zc = cconj(Zp);
     const float2 Ev = cscale(cadd(Z, Zc), 0.5f);
     const float2 Ov = cscale(cmul_mi(csub(Z, Zc)), 0.5f);
-    col[(size_t)k * I.lds] = (k == 0) ? make_float2(Ev.x + Ov.x, Ev.x - Ov.x) : cadd(Ev, cmul(s_tw[k], Ov));
+    col[(size_t)k * lds] = (k == 0) ? make_float2(Ev.x + Ov.x, Ev.x - Ov.x) : cadd(Ev, cmul(s_tw[k], Ov));
     if (kp != k) {
       const float2 Zc2 = cconj(Z);
       const float2 Ev2 = cscale(cadd(Zp, Zc2), 0.5f);
       const float2 Ov2 = cscale(cmul_mi(csub(Zp, Zc2)), 0.5f);
-      col[(size_t)kp * I.lds] = cadd(Ev2, cmul(s_tw[kp], Ov2));
+      col[(size_t)kp * lds] = cadd(Ev2, cmul(s_tw[kp], Ov2));
     }
   }
 }
@@ -332,6 +342,7 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
   using C = ConvCfg<LOGL, BLOCK>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const RegInst& I = B.in[blockIdx.y];
+  const int lds = I.lds;
   const int N = I.N, Np = F::L;
   const int c = threadIdx.x / F::TT, t = threadIdx.x % F::TT;
   float2* s_tw1 = reinterpret_cast<float2*>(smem_raw) + C::CT * C::SMV;
@@ -353,7 +364,7 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
     const int j = e % F::L, ci = e / F::L, it = item_of(2 * ci);
     float2* dst = reinterpret_cast<float2*>(smem_raw) + 2 * ci * C::SMV + pad32(j);
     const bool ok = it <= Np && j < N;
-    cp_async8(dst, I.S + (size_t)(ok ? slot_of(it) : 0) * I.lds + (ok ? j : 0), ok);
+    cp_async8(dst, I.S + (size_t)(ok ? slot_of(it) : 0) * lds + (ok ? j : 0), ok);
   }
   cp_async_commit();
   cp_async_wait_all();
@@ -361,7 +372,7 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
 
   const int item = item_of(c), h = c & 1;
   float2* sm = reinterpret_cast<float2*>(smem_raw) + c * C::SMV;
-  const float* lam = I.lreg + ((size_t)kx_of(item) * 2 + h) * Np;
+  const float* lam = I.sym + ((size_t)kx_of(item) * 2 + h) * Np;
   float2 x[F::E];
   // both halves read the column from the even vector's buffer; the barrier
   // keeps the even half's transform from overwriting it before the odd half
@@ -400,7 +411,7 @@ __global__ void __launch_bounds__(BLOCK, ConvCfg<LOGL, BLOCK>::kBlocksPerSm) kr_
     const int it = item_of(2 * i);
     if (it > Np || it == 1) continue;
     const float2* se = base + (2 * i) * C::SMV;
-    float2* col = I.S + (size_t)slot_of(it) * I.lds;
+    float2* col = I.S + (size_t)slot_of(it) * lds;
     for (int j = threadIdx.x; j < N; j += BLOCK) {
       const float2 w = twh[j];
       const float2 y = cadd(se[pad32(j)], cmulc(se[C::SMV + pad32(j)], w));
@@ -423,6 +434,7 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   using C = RowCfg<LOGL, BLOCK>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const RegInst& I = B.in[blockIdx.y];
+  const int lds = I.lds;
   const int N = I.N, Np = F::L;
   if ((int)blockIdx.x * C::VB >= N) return;
   const int v = threadIdx.x / F::TT, t = threadIdx.x % F::TT;
@@ -467,7 +479,7 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
     const float2* col = I.S + (ok ? row0 + vv : 0);
     float2* dst = base + vv * C::SMV;
     for (int k = threadIdx.x / C::VB; k < F::L; k += BLOCK / C::VB)
-      cp_async8(&dst[pad32(k)], col + (ok ? (size_t)k * I.lds : 0), ok);
+      cp_async8(&dst[pad32(k)], col + (ok ? (size_t)k * lds : 0), ok);
   }
   cp_async_commit();
   cp_async_wait_all();
@@ -511,6 +523,7 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   // (C + conv/2 = -kappa tau L_h u~; d = 0 at n = 0).
   const float tau = I.tau, tau2 = I.tau2;
   const size_t rbase = (size_t)rrow * I.ld;
+  const float* Frow = I.F ? I.F + (size_t)rrow * I.ldF : nullptr;
   // the equation is uniform over the launch: one loop per equation, so the
   // wave step's loop carries nothing of the diffusion step's
   auto bn_loop = [&](auto diff_c) {
@@ -554,13 +567,13 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
             const float u = e ? uv[j2].y : uv[j2].x;
             if constexpr (!DIFF) {
               float gs = g_of_r(I, u);
-              if (I.F) gs += I.fsc * I.F[(size_t)rrow * I.ldF + x];
+              if (I.F) gs += I.fsc * Frow[x];
               const float gg = tau2 * gs;
               b[e] = I.first ? tau * I.phi2[rbase + x] + 0.5f * (c + gg) : c + gg;
             } else {
               const float d = e ? dv[j2].y : dv[j2].x;
               float gs = g_of_r(I, u + 0.5f * d);
-              if (I.F) gs += I.fsc * I.F[(size_t)rrow * I.ldF + x];
+              if (I.F) gs += I.fsc * Frow[x];
               b[e] = (c + 0.5f * cx) + tau2 * gs - d;
             }
           }
@@ -611,14 +624,14 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
   store_nat<LOGL>(x, sm, t);
   __syncwarp();
   if (!valid) return;   // uniform over the row's threads, one part of a warp
-  float y[F::E];
-  gs_out_reg<LOGL>(y, sm, t, I, [] { __syncwarp(row_mask<F::TT>()); });
+  const int r = I.r;
+  if (r > 0) gs_border_reg<LOGL>(sm, t, I, [] { __syncwarp(row_mask<F::TT>()); });
   float* wrow = I.W + (size_t)row * I.ld;
-  static_for<0, F::E>([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
+#pragma unroll 2
+  for (int q = 0; q < F::E; ++q) {
     const int k = t + F::TT * q;
-    if (k < N) wrow[k] = y[q];
-  });
+    if (k < N) wrow[k] = gs_out_reg<LOGL>(sm, k, r);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -678,15 +691,15 @@ __global__ void __launch_bounds__(BLOCK, 3) kr_cols_solve(const __grid_constant_
   store_nat<LOGL>(x, sm, t);
   cp_async_wait_all();
   __syncthreads();
-  float y[F::E];
-  gs_out_reg<LOGL>(y, sm, t, I, [] { __syncthreads(); });
+  const int r = I.r;
+  if (r > 0) gs_border_reg<LOGL>(sm, t, I, [] { __syncthreads(); });
   if (!valid) return;
   const int first = I.first;
-  static_for<0, F::E>([&](auto qc) {
-    constexpr int q = decltype(qc)::value;
+#pragma unroll 2
+  for (int q = 0; q < F::E; ++q) {
     const int j = t + F::TT * q;
     if (j < N) {
-      const float uh = y[q];
+      const float uh = gs_out_reg<LOGL>(sm, j, r);
       // compensated leapfrog: d^{n+1} = d^n + uhat (d^1 = uhat), u^{n+1} = u^n + d^{n+1}
       // with u = u_hi + u_lo kept as a double-float pair (two-sum)
       const float d = first ? uh : s_d[j * C::CT + c] + uh;
@@ -701,7 +714,7 @@ __global__ void __launch_bounds__(BLOCK, 3) kr_cols_solve(const __grid_constant_
       I.u_lo[idx] = l2 - (h2 - s);
       I.u_d[idx] = d;
     }
-  });
+  }
 }
 
 constexpr int kRowBlock = 128;
