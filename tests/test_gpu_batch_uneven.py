@@ -37,6 +37,12 @@ def _make(S, prec_name, members):
 CASES = {
     # clusters of two blocks: 32 / 33 border columns, none, one, and many
     "gs-1024": ("SADI_PREC_FP32", [(1023, 1.0), (1024, 1.0), (991, 0.7), (992, 1.3), (600, 1.0)]),
+    # dense sweeps from r = 33 on (large kappa: H^-1 held whole, else I + E),
+    # the transforms' sweeps with the border inline up to r = 32
+    "gs-512": ("SADI_PREC_FP32", [(300, 1.0), (400, 900.0), (479, 0.7), (480, 1.0), (511, 1.3)]),
+    "gs-256": ("SADI_PREC_FP32", [(129, 900.0), (223, 1.0), (224, 1.0), (255, 0.7), (256, 1.0)]),
+    "gs-128": ("SADI_PREC_FP32", [(65, 1.0), (80, 900.0), (95, 0.7), (96, 1.0), (127, 1.3), (128, 1.0)]),
+    "dense-1024": ("SADI_PREC_FP32_DENSE", [(1023, 1.0), (600, 1.0), (1024, 0.7)]),
     # clusters of eight
     "dense-2048": ("SADI_PREC_FP32_DENSE", [(2047, 1.0), (2048, 1.0), (2041, 0.7), (1990, 1.3)]),
 }
