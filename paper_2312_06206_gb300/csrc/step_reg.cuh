@@ -596,7 +596,8 @@ __global__ void __launch_bounds__(BLOCK, RowCfg<LOGL, BLOCK>::kMinBlocks) kr_row
             float* wr = I.W + rbase;
             if (x + 1 < N) *reinterpret_cast<float2*>(wr + x) = make_float2(b[0], b[1]);
             else wr[x] = b[0];
-            if (I.Bh) {
+            // (none where dense sweeps follow in FP32, which N' = 1024 never takes)
+            if (LOGL == 10 || I.Bh) {
               unsigned hi, lo;
               split_bf16x2(b[0], b[1], &hi, &lo);
               *reinterpret_cast<unsigned*>(I.Bh + (size_t)rrow * I.ldp + x) = hi;
