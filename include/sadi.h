@@ -178,13 +178,15 @@ sadi_status sadi_set_initial(sadi_ctx *ctx, const double *phi1, const double *ph
 sadi_status sadi_step(sadi_ctx *ctx, int nsteps);
 
 /* Advance each of count contexts by nsteps time steps (asynchronous), as
- * sadi_step would, but batched: FP32 and FP32_DENSE contexts (unless explicit
- * tiles keep them on the shared-memory engine, see sadi_set_tiles) are grouped
- * by precision and N' (at most 32 per group) and each
+ * sadi_step would, but batched: FP32 contexts with FFT length N' <= 1024 and
+ * FP32_DENSE contexts with N' <= 2048 (unless explicit tiles keep them on
+ * the shared-memory engine, see sadi_set_tiles) are grouped by precision and
+ * N' (at most 32 per group; FP32 at N' <= 512 also by whether the border rank
+ * N' - N exceeds 32) and each
  * group runs one launch per kernel for all its members (independent problems
  * of possibly different N, alpha, kappa, tau and g; both dense sweeps of up
- * to 8 members in one GEMM launch); the other contexts step one after
- * another.
+ * to 8 members in one GEMM launch).  Other FP32_DENSE contexts of one N' share
+ * their GEMM launches; the other contexts step one after another.
  * All contexts must be initialised and distinct (SADI_EINVAL / SADI_ESTATE
  * otherwise).  The work
  * is issued on the first context's stream, ordered after the work already
@@ -284,9 +286,10 @@ void sadi_graph_destroy(sadi_graph *graph);
  * sadi_batch_step steps it (up to 32 contexts per group) -- SADI_PREC_FP32
  * (Gohberg-Semencul FFT sweeps) and, unless flags bit 0 is set or
  * s a_0 > 0.2 (the dense form's accuracy limit above),
- * SADI_PREC_FP32_DENSE (tensor-core dense-inverse sweeps) -- and, for FP32 at
- * N' > 1024, beside the default engine the shared-memory engine with the work
- * decomposition of sadi_set_tiles by coordinate descent.  flags bit 1 keeps the precision the
+ * SADI_PREC_FP32_DENSE (tensor-core dense-inverse sweeps) -- and, for a
+ * form on the shared-memory FFT engine (FP32 at N' > 1024, FP32_DENSE at
+ * N' > 2048), the work decomposition of sadi_set_tiles by coordinate
+ * descent.  flags bit 1 keeps the precision the
  * contexts already have (FP32 or FP32_DENSE, equal within each N) and tunes
  * only the tiles.  Each context is left with g, the fastest precision and
  * tiles of its group, uninitialised (call sadi_set_initial next).  Must precede sadi_set_initial and
@@ -349,20 +352,22 @@ sadi_status sadi_get_info(const sadi_ctx *ctx, int *fft_len, int *border_rank);
  * selected: grid rows per block of the row kernels, spectrum slots per block
  * of the column convolution (a divisor of N'), grid columns per block of the
  * y sweep.  conv_cols = -1 selects the three-pass column convolution (a
- * four-step FFT through HBM; FP32 forms, N' = 2048 .. 8192; its buffers, about
- * 24 N'^2 bytes, are allocated on first use).
+ * four-step FFT through HBM; FP32 forms, N' = 2048 .. 8192; the default at
+ * N' = 8192; its buffers, about 24 N'^2 bytes, are allocated on first use).
  * All zero restores the defaults.  Invalid combinations (shared memory above
  * 227 KB per block, more rows than the row kernel stages, -1 elsewhere)
  * return SADI_EINVAL and leave the setting unchanged.  The tiles change the
  * order of some rounding steps (the column convolution multiplies the symbol
  * fused into its transforms or in a separate pass), so results of different
  * tiles agree to rounding, not bitwise.  The tiles are those of the
- * shared-memory FFT engine, which runs FP64 and, from N' = 2048 on, an FP32
- * form given explicit (non-zero) tiles; by default the FP32 forms run on the
- * register paths, which have none (all zero moves a context back).  For
- * FP32_DENSE at N' = 2048 a change of the engine must precede
- * sadi_set_initial and sadi_set_source (SADI_ESTATE otherwise).  Call after
- * sadi_set_options. */
+ * shared-memory FFT engine: FP64, FP32 from N' = 2048 and FP32_DENSE from
+ * N' = 4096 on.  The register paths (FP32 at N' <= 1024, FP32_DENSE at
+ * N' <= 2048) and the dense products of FP64 at N' <= 128 have none.  At
+ * N' = 2048 explicit (non-zero) tiles move the dense form's FFT part to the
+ * shared-memory engine (all zero moves it back); such a change must precede
+ * sadi_set_initial and sadi_set_source (SADI_ESTATE otherwise).  Tiles other
+ * than the defaults move FP64 at N' <= 128 to the transforms of that engine.
+ * Call after sadi_set_options. */
 sadi_status sadi_set_tiles(sadi_ctx *ctx, int rows, int conv_cols, int solve_cols);
 
 /* Current tiles of the selected precision: tiles[0..2] = rows, conv_cols,

@@ -102,19 +102,20 @@ int slot_rows(int N) { return (N + 7) / 8 * 8; }
 
 size_t esize(int prec) { return prec == SADI_PREC_FP64 ? sizeof(double) : sizeof(float); }
 
-// The FFT engine of the context's precision: the register paths for both FP32
-// forms, except that explicit tiles, which the shared-memory engine alone
-// has, select that engine from N' = 2048 on.
+// The FFT engine of the context's precision: a register path where one serves
+// the form and length (both FP32 forms up to N' = 1024, the dense form's FFT
+// part up to N' = 2048), else the shared-memory engine.  Explicit tiles, which
+// that engine alone has, select it for the dense form at N' = 2048.
 bool wants_reg_path(const sadi_ctx* c) {
   if (!reg_path_supported(c->g.logNp, c->prec)) return false;
   return !(c->tiles_explicit && c->g.logNp >= kTilesMinLog);
 }
 
-// Tables of the direct path for the context's precision (see dir_mode).
-// whether the direct path holds H^-1 as I + E: while the ADI factor I + s T is
+// Whether the direct path holds H^-1 as I + E: while the ADI factor I + s T is
 // within 1/2 of the identity in its diagonal, s a_0 <= 1/2 (a_0 < 2.01 for
 // every alpha; H^-1 = I + E then has no cancellation in B + B E)
 bool dir_ident(const sadi_ctx* c) { return 2.0 * c->s <= 0.5; }
+// Tables of the direct path for the context's precision (see dir_mode).
 template <typename T>
 sadi_status build_direct(sadi_ctx* c, int mode) {
   const size_t N = c->g.N;
@@ -661,8 +662,8 @@ bool uses_direct64(const sadi_ctx* c) { return c->prec == SADI_PREC_FP64 && c->d
 bool uses_reg_path(const sadi_ctx* c) { return c->prec == SADI_PREC_FP32 && c->reg_path; }
 bool is_dense(const sadi_ctx* c) { return c->prec == SADI_PREC_FP32_DENSE; }
 
-// One step of a context on the shared-memory engine (FP64, or FP32 N' > 1024),
-// on stream st.
+// One step of a context on the shared-memory engine (FP64, or FP32 N' > 1024)
+// or, FP64 at N' <= 128, on the direct path, on stream st.
 sadi_status step_smem(sadi_ctx* c, cudaEvent_t* ev, cudaStream_t st) {
   const RhsParams rp = rhs_of(c, c->n);
   cudaError_t e;
@@ -1145,7 +1146,7 @@ sadi_status sadi_set_tiles(sadi_ctx* c, int rows, int conv_cols, int solve_cols)
   if (dflt) t = f64 ? default_tiles<double>(c->g.Np, c->g.N) : default_tiles<float>(c->g.Np, c->g.N);
   const bool ok = f64 ? tiles_valid<double>(c->g, t) : tiles_valid<float>(c->g, t);
   if (!ok) return fail(c, SADI_EINVAL, "tile sizes invalid for this N and precision");
-  // the engine these tiles select (from N' = 2048 on: explicit tiles the
+  // the engine these tiles select (dense form at N' = 2048: explicit tiles the
   // shared-memory engine, the defaults the register path; both keep the state
   // in the same layout); the FP64 path's tiles leave the FP32 forms' choice
   // alone

@@ -38,8 +38,8 @@ struct sadi_ctx {
   double2* stw64 = nullptr;  // per-stage FFT twiddles
   float2* stw32 = nullptr;
   Tiles tiles64{}, tiles32{};
-  // tiles set explicitly (not the defaults): from N' = 2048 on they select
-  // the shared-memory engine for the FP32 forms
+  // tiles set explicitly (not the defaults): at N' = 2048 they keep the
+  // dense form on the shared-memory engine
   bool tiles_explicit = false;
   // FP32 register-FFT path tables
   float2* rtw1 = nullptr;
@@ -103,7 +103,7 @@ struct sadi_ctx {
   int* tcerr = nullptr;             // device flag: a bounded wait in a GEMM ran out
   long long dbg_expire_ns = 0;      // sadi_debug_expire_waits: next dense step's waits run out (0: off)
   int* tcdep = nullptr;             // per 128-column panel: x-sweep tiles stored (zeroed each step)
-  sadi::Conv3 c3;                   // explicit tiles with conv_cols = -1: three-pass column convolution
+  sadi::Conv3 c3;                   // FP32 forms with conv_cols = -1 (N' = 8192): three-pass column convolution
   std::unique_ptr<TcInst> tc_x, tc_y;
   std::string tune_log;             // choice of sadi_autotune
   // state watchdog: after a stepping call in which n reaches a multiple of
