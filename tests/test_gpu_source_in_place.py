@@ -18,7 +18,8 @@ def env():
     from paper_2312_06206_gb300 import build
     build.build()
     from paper_2312_06206_gb300 import sadi
-    return sadi, torch
+    yield sadi, torch
+    torch.cuda.empty_cache()      # later tests measure and bound allocations
 
 
 @pytest.mark.parametrize("equation", ["wave", "diffusion"])
