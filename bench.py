@@ -339,10 +339,10 @@ def aggregate(times, world_size, pts_per_step, steps_list, reduce_max=None):
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of a
 # kernel in a workload, from the ncu captures summarised under profiles/
-# (kr_rows_r2c_n1023.md, kr_cols_conv_n1023.md, kr_rows_solve_dense_n1023.md,
+# (kr_rows_r2c_n1023.md, kb_cols_conv_n1023.md, kr_rows_solve_dense_n1023.md,
 # k_tc_gemm_n1023.md, k_tc_gemm_n4095.md); absent = no capture of the
 # current kernel, reported as null.
-NCU_TRAFFIC = {("n1023", "kr_rows_r2c"): 12.66e6, ("n1023", "kr_cols_conv"): 50.48e6,
+NCU_TRAFFIC = {("n1023", "kr_rows_r2c"): 12.66e6, ("n1023", "kr_cols_conv"): 37.85e6,   # kb_cols_conv
                ("n1023", "kr_rows_solve<dense>"): 70.76e6, ("n1023", "k_tc_gemm(x+y)"): 89.4e6,
                ("n4095", "k_tc_gemm(x+y)"): 1733.6e6}
 
@@ -412,10 +412,10 @@ def roofline_of(phase_ms, N, Np, dense, ninst, workload):
     kernel's bound is the roof its algorithmic intensity (method flops per
     method byte) meets first: HBM below the ridge FP32 peak / HBM peak, the
     FP32 pipes above it; a kernel with no method flops is HBM-bound."""
-    # the phases' labels, by the kernels of the shared-memory engine and of the
-    # register path up to N' = 1024 (the dense form's FFT part: 2048); the block
-    # path (kb_rows_r2c, kb_cols_conv*, kb_rows_solve, kb_cols_solve) reports
-    # its phases under the same labels
+    # the phases' labels, by engine: shared-memory engine, or register paths up
+    # to N' = 1024 (the dense form's FFT part: 2048).  "runs" names the kernel:
+    # from N' = 256 on the block path's (kb_*), but for the dense form's row
+    # kernels at 1024
     reg = Np <= 1024 or (dense and Np == 2048)
     pre = "kr_" if reg else "k_"
     conv = "kr_cols_conv" if reg else ("k_conv3_a+b+c" if Np == 8192 else "k_cols_conv")   # three passes at 8192
@@ -424,6 +424,11 @@ def roofline_of(phase_ms, N, Np, dense, ninst, workload):
     else:
         ysweep = "kr_cols_solve" if reg else "k_transpose+k_rows_gs+k_transpose_leapfrog"
         names = [pre + "rows_r2c", conv, pre + "rows_solve", ysweep]
+    runs = list(names)
+    if reg and Np >= 256:
+        runs[1] = "kb_cols_conv_seq" if Np == 2048 else "kb_cols_conv"
+        if not (dense and Np == 1024):
+            runs = [r.replace("kr_", "kb_") for r in runs]
     alg = algorithmic(N, Np, dense)
     pk = peaks_of()
     fp32_peak, hbm_peak, bf16_peak = pk["fp32_tflops"], pk["hbm_gbs"], pk["bf16_tflops_sustained"]
@@ -437,7 +442,7 @@ def roofline_of(phase_ms, N, Np, dense, ninst, workload):
         gbs = b_alg * ninst / dur / 1e9
         tfl = None if f_alg is None else f_alg * ninst / dur / 1e12
         ach, peak, unit = (gbs, hbm_peak, "GB/s") if bound == "hbm" else (tfl, fp32_peak, "TFLOP/s")
-        e = {"us": phase_ms[k] * 1e3, "share": phase_ms[k] / sum(phase_ms), "bound": bound,
+        e = {"runs": runs[k], "us": phase_ms[k] * 1e3, "share": phase_ms[k] / sum(phase_ms), "bound": bound,
              "intensity_flop_per_byte": inten, "achieved": ach, "peak": peak, "unit": unit, "frac": ach / peak,
              "hbm_gbs": gbs, "hbm_frac": gbs / hbm_peak, "fp32_tflops": tfl,
              "alg_bytes": b_alg * ninst, "alg_flops": None if f_alg is None else f_alg * ninst,

@@ -1,9 +1,11 @@
-"""The block-FFT path of the FP32 forms (FFT lengths 2048 .. 8192) against the
-shared-memory engine (explicit tiles) and the FP64 path, at the sizes where its
-clusters of eight rows, its slot runs and its border correction change: the
-smallest N of a length, N one above and below a multiple of eight, border ranks
-32 (added inside the sweep kernels), 33 and 1023 (one product per sweep), and
-N = N' (no border).
+"""The FP32 forms on the engines and lengths around the block-FFT path, which
+serves FFT lengths 256 .. 1024 (GS form) and 256 .. 2048 (dense form), against
+the shared-memory engine (explicit tiles), which runs the longer ones, and
+against the FP64 path: at the smallest N of a length, N one above and below a
+multiple of eight, border ranks around 32, and N = N' (no border).  Where a form
+has one engine (GS from N' = 2048, dense from 4096 on) the two runs of the engine
+comparisons are the same engine; batches of uneven border ranks at the lengths
+that batch them are in test_gpu_batch_uneven.py.
 
 Tolerances: both engines compute the same FP32 transforms in different orders.
 One transform of length L carries a relative error of about eps log2 L
